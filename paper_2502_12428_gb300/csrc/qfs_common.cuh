@@ -1,4 +1,4 @@
-// Definitions shared by the per-quartic pipeline (qfs_engine.cuh) and the swept chain product (qfs_sweep.cuh):
+// Definitions shared by the per-quartic pipeline (qfs_engine.cuh) and the chain products (qfs_sweep.cuh, qfs_block.cuh):
 // block size, device status bits, debug outputs and the static part of the shared memory.
 #pragma once
 #include <cstddef>
@@ -9,6 +9,7 @@ namespace qfs {
 
 constexpr int kThreads = 256;
 constexpr int kMaxUparDecl = 8;
+constexpr int kMaxStrips = 100;   // strips of a block product (qfs_block.cuh)
 
 // Workspace buffers.  Every buffer a chain product reads from is preceded by kGuardWords zero words (the swept
 // product reads columns that do not exist from there).  A launch's workspace holds, per CTA, two buffers of
@@ -44,12 +45,19 @@ struct DebugPtrs {
 struct Smem {
   int SW[kSWLen];
   int taps[35];           // coefficients of f, packed order (index tet(uI) + tri(sI) + tI)
-  uint32_t tapword[15];   // dp4a tap words per (uI, sI) pair: byte k = a(uI, sI, 3-k)
+  uint32_t tapword[15];   // tap words per (uI, sI) pair: byte k = a(uI, sI, 3-k)
   uint32_t pair_mask;     // bit tri(uI)+sI set iff that pair has a nonzero tap
   int dense_min;          // nonzero tap pairs from which the swept chain runs every pair (the two-slice loop)
   int powp[kMaxP];        // c^p mod p^2
   int slot_tab[2][kMaxUparDecl + 4];  // ring word offsets of the slices a chain round reads (double buffered)
-  uint16_t chunk_tab[32 * 40];        // chain block: flat chunk index -> (column - s0) << 8 | chunk
+  union {                             // one product form per launch
+    uint16_t chunk_tab[32 * 40];      // slice ring: flat chunk index -> (column - s0) << 8 | chunk
+    struct {                          // block products
+      uint32_t strip_tab[kMaxStrips]; // first item of every strip (block::build_strip_tab)
+      int unit_next[2];               // next unit of a product's queue, by the product's parity
+      int unit_slot[4][2];            // a team's next unit
+    };
+  };
   int tile_round, tile_ring;          // chain tile configuration of the current quartic's prime
   int64_t item;
   int flag;

@@ -21,6 +21,7 @@
 #include "qfs_layout.cuh"
 #include "qfs_common.cuh"
 #include "qfs_sweep.cuh"
+#include "qfs_block.cuh"
 
 namespace qfs {
 
@@ -97,12 +98,11 @@ __host__ __device__ inline int chain_slot_words(int p, TileConfig tc) {
 __host__ __device__ inline int theta_ring_words_for(int p, int power = -1);
 
 // Ring words the identity and reduced power modes need: three byte arrays (f^(p-2), Delta_1(f), E), and in the
-// reduced mode a product to degree 4p whose own slot ring (int8 tensor form only) starts after f^(p-2),
-// Delta_1(f) and q.
+// reduced mode a product to degree 4p whose own ring starts after f^(p-2), Delta_1(f) and q.
 __host__ __device__ inline int aux_ring_words(int p, TileConfig tc, bool ring_chain) {
   const int l_fpm2 = tet(4 * (p - 2) + 1), l_d1f = tet(4 * p + 1), l_E = tet(4 * (p - 1) + 1);
   const int ring_off = (((l_fpm2 + l_d1f + 3) / 4 + 64) + 3) & ~3;
-  int chain = 0;
+  int chain = block_ring_words(p);
   if (ring_chain)
     for (int s0 = 0; s0 <= 4 * p; s0 += 32) {
       const ChainTile T = chain_tile(s0, 4 * p, tc);
@@ -112,15 +112,15 @@ __host__ __device__ inline int aux_ring_words(int p, TileConfig tc, bool ring_ch
 }
 
 // Which chain product a form runs at prime p: the shared-memory slice ring (the int8 tensor form, whose tiles read
-// aligned words of a staged slice), or the lane sweep over global memory (dp4a and int32 forms).
+// aligned words of a staged slice), or one that needs no more than block_ring_words (dp4a and int32 forms).
 __host__ __device__ constexpr bool uses_ring_chain(int form, int p) { return form == 2 && p > 0; }
 
-// Shared-memory ring words for prime p: the chain's slice ring (when the chain stages slices in shared memory),
+// Shared-memory ring words for prime p: the chain's slice ring (the int8 tensor form's, or the dp4a form's strips),
 // theta's Delta slots, and the power modes' arrays.  ring_chain = true gives the size every form fits in;
 // power (QFS_POWER_*, -1 for every mode) sizes theta for one power mode.
 __host__ __device__ inline int ring_words_for(int p, TileConfig tc, bool ring_chain = true, int power = -1) {
-  return max(max(ring_chain ? chain_slot_words(p, tc) : 0, theta_ring_words_for(p, power)),
-             aux_ring_words(p, tc, ring_chain));
+  return max(max(max(ring_chain ? chain_slot_words(p, tc) : 0, block_ring_words(p)), theta_ring_words_for(p, power)),
+             power != 0 ? aux_ring_words(p, tc, ring_chain) : 0);
 }
 
 __host__ __device__ inline size_t smem_bytes_for(int p, TileConfig tc, bool ring_chain = true) {
@@ -129,13 +129,6 @@ __host__ __device__ inline size_t smem_bytes_for(int p, TileConfig tc, bool ring
 __host__ __device__ inline size_t smem_bytes_for(int p, bool ring_chain = true) {
   return smem_bytes_for(p, default_tile(p), ring_chain);
 }
-
-__device__ __forceinline__ void cp_async16(uint32_t *smem, const uint32_t *gmem, bool valid) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem), "r"(valid ? 16 : 0));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::); }
 
 namespace detail {
 
@@ -468,16 +461,18 @@ __device__ __forceinline__ void ring_chain_step(const uint32_t *__restrict__ in,
   if (bad) atomicOr(status, kStatusInexactDivision);
 }
 
-// One product of the chain: over the shared-memory slice ring above (int8 tensor form), or lane by lane over the
-// input slices in global memory (qfs_sweep.cuh; dp4a and int32 forms).
+// One product of the chain: over the shared-memory slice ring above (int8 tensor form), by strips and blocks of slices
+// (qfs_block.cuh; dp4a form), or lane by lane over the input slices in global memory (qfs_sweep.cuh; int32 form).
 template <int P, int FORM, bool LAST, bool DEBUG>
 __device__ __forceinline__ void chain_step(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, int m_in,
                                            Smem &sm, uint32_t *ring, const uint8_t *gs, uint32_t *status,
                                            DebugPtrs dbg) {
   if constexpr (uses_ring_chain(FORM, P))
     ring_chain_step<P, FORM, LAST, DEBUG>(in, out, m_in, sm, ring, gs, status, dbg);
+  else if constexpr (FORM == 1)
+    block_chain_step<P, LAST, DEBUG>(in, out, m_in, sm, ring, gs, status, dbg);
   else
-    sweep_chain_step<P, FORM, LAST, DEBUG>(in, out, m_in, sm, gs, status, dbg);
+    sweep_chain_step<P, LAST, DEBUG>(in, out, m_in, sm, gs, status, dbg);
 }
 
 // ------------------------------------------------------------------------------------------------ theta
@@ -1140,6 +1135,8 @@ __device__ __forceinline__ bool setup_quartic(const uint8_t *__restrict__ f35, S
     bad = a >= P;
     sm.taps[tid] = a;
   }
+  block::build_strip_tab(P, sm);
+  if (tid < 2) sm.unit_next[tid] = 0;
   if (__syncthreads_or(bad)) return false;
   if (tid == 0) {
     uint32_t mask = 0;

@@ -114,6 +114,39 @@ def test_stages_p11(qfs):
         assert np.array_equal(got["iters"].cpu().numpy()[:1], it["iters"])
 
 
+def _edge_quartics(p):
+    """x4^4 plus each other monomial in turn (one tap beside tap (4, 4, 4): every tap position of the products'
+    windows), every coefficient p - 1 (the largest sums), and two taps at the ends of one window."""
+    rows = []
+    for k in range(34):
+        f = np.zeros(35, np.uint8)
+        f[k], f[34] = p - 1, 1
+        rows.append(f)
+    rows.append(np.full(35, p - 1, np.uint8))
+    f = np.zeros(35, np.uint8)
+    f[30], f[34] = p - 1, p - 1
+    rows.append(f)
+    return rows
+
+
+@pytest.mark.parametrize("p,step", [(3, 1), (5, 5), (7, 12)])
+def test_dp4a_product_tap_positions(qfs, p, step):
+    # G = f~^(p(p-1)) mod p^2 and Delta element by element, on quartics whose taps sit alone in the dp4a windows
+    rows = _edge_quartics(p)
+    rows = rows[:-2:step] + rows[-2:]
+    seen = 0
+    for f in rows:
+        ref = oracle.stage_arrays_fchain(p, f)
+        got = qfs.debug_stages(p, dev_tensor(f), max_h=2)
+        assert np.array_equal(got["g"].cpu().numpy(), ref["g"])
+        if got["h"] != 1:
+            seen += 1
+            assert np.array_equal(got["G"].cpu().numpy(), ref["D"])
+            assert np.array_equal(got["delta"].cpu().numpy(), ref["delta"])
+    assert seen >= len(rows) // 2
+    assert qfs.read_status() == 0
+
+
 # ------------------------------------------------------------------------------------- heights, small sets
 @pytest.mark.parametrize("form", CORE_FORMS)
 def test_heights_p3_64_plus_fermat(qfs, form):
