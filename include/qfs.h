@@ -157,7 +157,8 @@ int qfs_sweep_autotune(int form, int p, int64_t n, const uint8_t *coeffs, int *b
 int qfs_shutdown(void);
 
 /* Copies the device status word of the current device's last launches into *status_out (0 = no check failed;
-   bit 0 = an exact division by p in Delta_1 found a remainder; bit 1 = the theta test saw an out-of-range value),
+   bit 0 = an exact division by p in Delta_1 found a remainder; bit 1 = the theta test saw an out-of-range value;
+   bit 2 = a bounded wait inside a kernel ran out, and that call's result is not valid),
    then clears it.  The word covers every launch since the last call, qfs_heights_noalloc's included (that entry
    point keeps its own word in its fixed array; this call ORs it in and clears it too).  Synchronises the current
    device. */
@@ -230,9 +231,10 @@ int qfs_theta_matrix(int p, int64_t n, const uint8_t *coeffs, uint8_t *M_out, cu
 
 /* Matrix multiplication mod p (the paper's Sec. 5 workload, square matrices mod 11): C = A B mod p.
    A: device, n x k uint8, row-major; B: device, k x m uint8, row-major; C: device, n x m uint8, row-major; values
-   in [0, p), 2 <= p <= 256 (p need not be prime); all caller-owned.  Exact: products accumulate in int32 on the
-   int8 tensor cores and are reduced mod p.  Stream-ordered; may grow a library scratch buffer ((n + m) x k bytes
-   rounded up) with cudaMalloc.  Returns QFS_OK or QFS_ERR_INVALID_P, QFS_ERR_INVALID_N, QFS_ERR_NULL,
+   in [0, p), 2 <= p <= 256 (p need not be prime); all caller-owned.  Exact: the fp8 tensor cores multiply small
+   integers that e4m3 holds exactly (two planes per matrix for p > 33), and float32 sums are reduced mod p before they
+   could leave the integers float32 holds exactly.  Stream-ordered; may grow a library scratch buffer ((n + m) x k
+   bytes rounded up, twice that for p > 33) with cudaMalloc.  Returns QFS_OK or QFS_ERR_INVALID_P, QFS_ERR_INVALID_N, QFS_ERR_NULL,
    QFS_ERR_NO_MEMORY, QFS_ERR_CUDA (nothing enqueued on error).  n = 0 or m = 0 is a no-op; k = 0 zeroes C. */
 int qfs_matmul_mod(int p, int n, int m, int k, const uint8_t *A, const uint8_t *B, uint8_t *C, cudaStream_t stream);
 

@@ -758,7 +758,7 @@ extern "C" int qfs_matmul_mod(int p, int n, int m, int k, const uint8_t *A, cons
   DeviceState *S = nullptr;
   int rc = device_state(&S);
   if (rc) return rc;
-  const size_t need = matmul_scratch_bytes(n, m, k);
+  const size_t need = matmul_scratch_bytes(p, n, m, k);
   if (S->mm_bytes < need) {
     if (S->mm && cudaFree(S->mm) != cudaSuccess) return cuda_fail(cudaGetLastError());
     S->mm = nullptr;
@@ -769,7 +769,8 @@ extern "C" int qfs_matmul_mod(int p, int n, int m, int k, const uint8_t *A, cons
     }
     S->mm_bytes = need;
   }
-  cudaError_t e = matmul_mod_launch(p, n, m, k, A, B, C, static_cast<uint8_t *>(S->mm), stream);
+  cudaError_t e = matmul_mod_launch(p, n, m, k, A, B, C, static_cast<uint8_t *>(S->mm), S->sms,
+                                    reinterpret_cast<uint32_t *>(static_cast<char *>(S->ctrl) + 8), stream);
   return e == cudaSuccess ? QFS_OK : cuda_fail(e);
 }
 

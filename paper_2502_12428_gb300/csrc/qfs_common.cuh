@@ -34,6 +34,7 @@ __device__ __forceinline__ void cta_buffers(uint32_t *ws, size_t stride, uint32_
 // Status bits (atomicOr into the device status word).
 constexpr uint32_t kStatusInexactDivision = 1u;
 constexpr uint32_t kStatusTheta = 2u;
+constexpr uint32_t kStatusWait = 4u;   // a bounded wait inside a kernel ran out
 
 struct DebugPtrs {
   uint32_t *G;        // padded, degree D: raw G (mod p^2) before the Delta_1 epilogue

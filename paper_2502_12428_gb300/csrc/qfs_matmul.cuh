@@ -6,10 +6,11 @@
 
 namespace qfs {
 
-// scratch bytes qfs_matmul_mod needs for an (n x k) by (k x m) product
-size_t matmul_scratch_bytes(int n, int m, int k);
-// C = A B mod p (uint8 row-major, values in [0, p), 2 <= p <= 256); scratch: matmul_scratch_bytes(n, m, k) bytes
+// scratch bytes qfs_matmul_mod needs for an (n x k) by (k x m) product mod p
+size_t matmul_scratch_bytes(int p, int n, int m, int k);
+// C = A B mod p (uint8 row-major, values in [0, p), 2 <= p <= 256); scratch: matmul_scratch_bytes(p, n, m, k) bytes,
+// 1,024-byte aligned; sms: SMs of the device; status: device word that receives kStatusWait if a wait runs out
 cudaError_t matmul_mod_launch(int p, int n, int m, int k, const uint8_t *A, const uint8_t *B, uint8_t *C,
-                              uint8_t *scratch, cudaStream_t st);
+                              uint8_t *scratch, int sms, uint32_t *status, cudaStream_t st);
 
 }  // namespace qfs

@@ -509,6 +509,37 @@ def test_matmul_mod_matches_oracle(qfs, p, n, m, k):
     assert np.array_equal(got, oracle.matmul_mod(p, A, B))
 
 
+@pytest.mark.parametrize("p,n,m,k,lo", [
+    (33, 129, 257, 127, 0), (34, 129, 257, 129, 0),        # one e4m3 plane and two; edges of tiles and K steps
+    (33, 130, 260, 65536, 16), (33, 5, 9, 65664, 15),      # sums up to 2^24, and past one drain
+    (256, 127, 255, 896, 120), (251, 64, 300, 769, 112),   # the shortest drains, the largest plane products
+    (2, 1, 700, 4097, 0)])
+def test_matmul_mod_planes_and_drains(qfs, p, n, m, k, lo):
+    # whole values: any lost bit of an accumulation shows
+    rng = np.random.default_rng(p * 7 + k)
+    A = rng.integers(lo, min(p, lo + 18), (n, k), dtype=np.uint8)
+    B = rng.integers(lo, min(p, lo + 18), (k, m), dtype=np.uint8)
+    got = qfs.matmul_mod(p, dev_tensor(A), dev_tensor(B)).cpu().numpy()
+    want = (A.astype(np.int64) @ B.astype(np.int64)) % p
+    assert np.array_equal(got, want.astype(np.uint8))
+    assert qfs.read_status() == 0
+
+
+def test_matmul_mod_unaligned_views(qfs):
+    # row pitches and base addresses of every alignment: the pack reads and the product writes bytes then
+    rng = np.random.default_rng(77)
+    for off, n, m, k in [(0, 40, 16, 64), (1, 33, 24, 65), (2, 30, 20, 66), (3, 31, 37, 67)]:
+        A = rng.integers(0, 11, (n, k), dtype=np.uint8)
+        B = rng.integers(0, 11, (k, m), dtype=np.uint8)
+        bufs = [torch.zeros(x + 8, dtype=torch.uint8, device="cuda:0") for x in (n * k, k * m, n * m)]
+        a, b, c = (t[off:off + x].view(s) for t, x, s in zip(bufs, (n * k, k * m, n * m), ((n, k), (k, m), (n, m))))
+        a.copy_(torch.from_numpy(A))
+        b.copy_(torch.from_numpy(B))
+        qfs.matmul_mod(11, a, b, out=c)
+        assert np.array_equal(c.cpu().numpy(), oracle.matmul_mod(11, A, B))
+        assert not bufs[2][:off].any() and not bufs[2][off + n * m:].any()
+
+
 def test_matmul_mod_long_k_reduces_between_tiles(qfs):
     # k (p-1)^2 above 2^31 at p = 251: the accumulators are reduced between K tiles
     p, n, m, k = 251, 16, 24, 40000
