@@ -800,10 +800,7 @@ extern "C" int qfs_poly_power(int d, const uint32_t *coeffs, int n, uint32_t *ou
     S->pp_bytes = need;
   }
   uint32_t *scratch = static_cast<uint32_t *>(S->pp);
-  uint32_t *cdev = scratch + (need / sizeof(uint32_t) - n_in - 16);   // the input sits at the end of the scratch
-  cudaError_t e = cudaMemcpyAsync(cdev, coeffs, sizeof(uint32_t) * n_in, cudaMemcpyHostToDevice, stream);
-  if (e != cudaSuccess) return cuda_fail(e);
-  e = polypow_launch(d, n, nprimes, cdev, out, scratch, stream);
+  cudaError_t e = polypow_launch(d, n, nprimes, coeffs, out, scratch, stream);
   return e == cudaSuccess ? QFS_OK : cuda_fail(e);
 }
 

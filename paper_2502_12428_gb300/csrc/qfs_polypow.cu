@@ -76,21 +76,6 @@ __device__ __forceinline__ uint32_t mont_mul(uint32_t a, uint32_t b, const Prime
   return min(u, u - P.q);
 }
 
-// a = 0, then the packed input reduced mod q
-__global__ void zero_kernel(uint32_t *a, uint32_t N) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) a[i] = 0;
-}
-__global__ void scatter_kernel(const uint32_t *coeffs, int d, int B, uint32_t *a, PrimeQ P) {
-  const int n_in = tet(d + 1);
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_in; i += gridDim.x * blockDim.x) {
-    int u, s, t;
-    decode_packed(i, u, s, t);
-    // coefficient i belongs to the monomial with (u, s, t) = (e2+e3+e4, e3+e4, e4) in degree d
-    const int e2 = u - s, e3 = s - t, e4 = t;
-    a[(size_t)e2 + (size_t)B * e3 + (size_t)B * B * e4] = coeffs[i] % P.q;
-  }
-}
-
 // a w mod q for a < 2^32, w < q < 2^31, given ws = floor(w 2^32 / q) (Shoup): the quotient estimate
 // floor(a ws / 2^32) is at most one below floor(a w / q), so a w - est q lies in [0, 2q)
 __device__ __forceinline__ uint32_t shoup_mul(uint32_t a, uint32_t w, uint32_t ws, uint32_t q) {
@@ -111,6 +96,34 @@ constexpr int kMaxTableJobs = 3 * 2 * kPolyPowMaxPrimes;
 struct TableJobs {
   TableJob job[kMaxTableJobs];
 };
+// Twiddle tables of one prime and direction: lo[j] = w^j (j < 4096), hi[j] = w^(4096 j) (j < max(1, N / 4096)),
+// each with its Shoup companion, so that w^e = lo[e mod 4096] hi[e / 4096]; rt[j] = w_R^j (j < R / 2) for the
+// R-point transforms inside a pass, R = min(256, N), also with companions.
+struct TwTab {
+  const uint32_t *lo, *los, *hi, *his, *rt, *rts;
+};
+
+// What the kernels need of every prime; a launch takes the primes from the first on, one for each blockIdx.y, whose
+// transforms stand N words apart.  The pass kernels have an instance for a single prime (ONE), which finds its prime's
+// constants at fixed places of the parameter bank: n = 15, where the primes run one by one, took 1.88 ms with indexed
+// ones against 1.82.
+struct Primes {
+  PrimeQ P[kPolyPowMaxPrimes];
+  TwTab F[kPolyPowMaxPrimes], I[kPolyPowMaxPrimes];   // forward and inverse tables
+  uint32_t ninv[kPolyPowMaxPrimes], cn[kPolyPowMaxPrimes];   // N^-1 and 2^(32 n) mod q
+
+  Primes from(int j) const {   // the primes from j on
+    Primes R{};
+    for (int i = j; i < kPolyPowMaxPrimes; ++i) {
+      R.P[i - j] = P[i];
+      R.F[i - j] = F[i];
+      R.I[i - j] = I[i];
+      R.ninv[i - j] = ninv[i];
+      R.cn[i - j] = cn[i];
+    }
+    return R;
+  }
+};
 // Every power table of every prime and direction in one launch: blockIdx.y selects the table.
 __global__ void power_tables_kernel(TableJobs J) {
   const TableJob &T = J.job[blockIdx.y];
@@ -126,12 +139,32 @@ __global__ void power_tables_kernel(TableJobs J) {
   }
 }
 
-// Twiddle tables of one prime and direction: lo[j] = w^j (j < 4096), hi[j] = w^(4096 j) (j < max(1, N / 4096)),
-// each with its Shoup companion, so that w^e = lo[e mod 4096] hi[e / 4096]; rt[j] = w_R^j (j < R / 2) for the
-// R-point transforms inside a pass, R = min(256, N), also with companions.
-struct TwTab {
-  const uint32_t *lo, *los, *hi, *his, *rt, *rts;
+
+// The input, packed: every word of the leading rows of the transforms (the rest is never read), coefficients reduced
+// mod q.  One warp per run (e4, e3) of B words, lanes over e2.  Small inputs come with the launch (given), larger ones
+// from device memory.
+constexpr int kGivenCoeffs = 1024;
+struct GivenCoeffs {
+  uint32_t c[kGivenCoeffs];
 };
+__global__ void fill_kernel(const __grid_constant__ GivenCoeffs given, const uint32_t *coeffs, int d, int B,
+                            uint32_t cleared, uint32_t N, uint32_t *a, const __grid_constant__ Primes Q) {
+  const uint32_t q = Q.P[blockIdx.y].q;
+  a += (size_t)blockIdx.y * N;
+  const uint32_t *c = coeffs ? coeffs : given.c;
+  const int lane = threadIdx.x & 31;
+  const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+  for (uint32_t row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); (uint64_t)row * B < cleared; row += warps) {
+    const int e4 = (int)(row / (uint32_t)B), e3 = (int)(row % (uint32_t)B);
+    for (int e2 = lane; e2 < B; e2 += 32) {
+      const uint64_t i = (uint64_t)row * B + e2;
+      if (i >= cleared) break;
+      const int u = e2 + e3 + e4;
+      a[i] = u <= d ? c[tet(u) + tri(e3 + e4) + e4] % q : 0u;
+    }
+  }
+}
+
 constexpr int kTwLoBits = 12;
 constexpr int kPassMaxStages = 8;
 constexpr int kPassR = 1 << kPassMaxStages;   // longest column of a pass
@@ -254,8 +287,11 @@ __device__ __forceinline__ void load_root_table(uint32_t *rt, uint32_t *rts, con
 // column c times w_M^(c k), k = bitrev(m) (its frequency index).  Inverse: the twiddle w_M^(-c k) first, then the
 // R-point inverse DIT.  Each block takes kPassCols consecutive columns of one block of M.
 template <bool INV>
-__global__ void __launch_bounds__(256) ntt_column_pass(uint32_t *a, int logN, int logM, int kp, TwTab T,
-                                                       TwTab TR, PrimeQ P) {
+__global__ void __launch_bounds__(256) ntt_column_pass(uint32_t *a, int logN, int logM, int kp,
+                                                       const __grid_constant__ Primes Q) {
+  const PrimeQ P = Q.P[blockIdx.y];
+  const TwTab T = INV ? Q.I[blockIdx.y] : Q.F[blockIdx.y];
+  a += (size_t)blockIdx.y << logN;
   __shared__ uint32_t tile[kTileWords];
   __shared__ uint32_t rt[kPassR / 2], rts[kPassR / 2];
   __shared__ uint32_t p1[kPassCols][16], p2[kPassCols][16];
@@ -265,7 +301,7 @@ __global__ void __launch_bounds__(256) ntt_column_pass(uint32_t *a, int logN, in
   const uint32_t bb = q0 >> logNc, c0 = q0 & (Nc - 1);
   const size_t base = (size_t)bb * M + c0;
   constexpr int ld = kPassCols + 1;
-  load_root_table(rt, rts, TR, R, logN);
+  load_root_table(rt, rts, T, R, logN);
   column_twiddles(p1, p2, c0, logN - logM, T, P);
   if (INV) __syncthreads();
   for (int i = threadIdx.x; i < R * kPassCols; i += blockDim.x) {
@@ -296,8 +332,11 @@ __global__ void __launch_bounds__(256) ntt_column_pass(uint32_t *a, int logN, in
 
 // The innermost pass on contiguous runs of R = 2^kp elements: forward R-point DIF, every entry to the n-th power,
 // inverse R-point DIT.  A block takes G = min(N, kPassR kPassCols) / R runs.
-__global__ void __launch_bounds__(256) ntt_inner_pow(uint32_t *a, int logN, int kp, uint32_t n, TwTab TF,
-                                                     TwTab TI, PrimeQ P) {
+__global__ void __launch_bounds__(256) ntt_inner_pow(uint32_t *a, int logN, int kp, uint32_t n,
+                                                     const __grid_constant__ Primes Q) {
+  const PrimeQ P = Q.P[blockIdx.y];
+  const TwTab TF = Q.F[blockIdx.y], TI = Q.I[blockIdx.y];
+  a += (size_t)blockIdx.y << logN;
   __shared__ uint32_t tile[kTileWords];
   __shared__ uint32_t rf[kPassR / 2], rfs[kPassR / 2], ri[kPassR / 2], ris[kPassR / 2];
   const int R = 1 << kp;
@@ -410,9 +449,12 @@ __device__ __forceinline__ uint32_t column_twiddle(uint32_t x, const uint32_t *p
 // (row stride kPassCols + 1).
 // nz_rows (forward): rows m >= nz_rows of every column are zero and are not read (the first pass of a transform
 // whose input fills only its leading rows).
-template <int KP, bool INV>
-__global__ void __launch_bounds__(kNttThreads) ntt_column_regs(uint32_t *a, int logN, int logM, TwTab T, TwTab TR,
-                                                               PrimeQ P, int nz_rows) {
+template <int KP, bool INV, bool ONE>
+__global__ void __launch_bounds__(kNttThreads) ntt_column_regs(uint32_t *a, int logN, int logM,
+                                                               const __grid_constant__ Primes Q, int nz_rows) {
+  const PrimeQ &P = Q.P[ONE ? 0 : blockIdx.y];
+  const TwTab &T = INV ? Q.I[ONE ? 0 : blockIdx.y] : Q.F[ONE ? 0 : blockIdx.y];
+  a += (size_t)blockIdx.y << logN;
   static_assert(KP >= 2 && KP <= kPassMaxStages, "two register phases");
   constexpr int K1 = KP / 2, K2 = KP - K1, ld = kPassCols + 1;
   constexpr int NT1 = kPassCols << K2, NT2 = kPassCols << K1;   // tasks of the strided and the contiguous phase
@@ -424,7 +466,7 @@ __global__ void __launch_bounds__(kNttThreads) ntt_column_regs(uint32_t *a, int 
   const uint32_t q0 = blockIdx.x * kPassCols;
   const uint32_t bb = q0 >> logNc, c0 = q0 & (Nc - 1);
   uint32_t *col = a + ((size_t)bb << logM) + c0;
-  load_root_table(rt, rts, TR, 1 << KP, logN);
+  load_root_table(rt, rts, T, 1 << KP, logN);
   column_twiddles(p1, p2, c0, logN - logM, T, P);
   __syncthreads();
   if (!INV) {
@@ -522,8 +564,13 @@ __device__ __forceinline__ uint32_t pow_mont(uint32_t x, uint32_t n, uint32_t c,
 // DIT without leaving registers, then the strided phase of the inverse.  Shared tile: run g, element m at
 // g RW + (m >> K2) BW + (m mod 2^K2) with blocks padded to BW = 2^K2 + 1 words, so that both phases' accesses
 // (16 lanes per run, two runs per warp) are free of bank conflicts.  cn = 2^(32 n) mod q (pow_mont).
-__global__ void __launch_bounds__(kNttThreads) ntt_inner_regs(uint32_t *a, int logN, uint32_t n, uint32_t cn,
-                                                              TwTab TF, TwTab TI, PrimeQ P) {
+template <bool ONE>
+__global__ void __launch_bounds__(kNttThreads) ntt_inner_regs(uint32_t *a, int logN, uint32_t n,
+                                                              const __grid_constant__ Primes Q) {
+  const PrimeQ &P = Q.P[ONE ? 0 : blockIdx.y];
+  const TwTab &TF = Q.F[ONE ? 0 : blockIdx.y], &TI = Q.I[ONE ? 0 : blockIdx.y];
+  const uint32_t cn = Q.cn[ONE ? 0 : blockIdx.y];
+  a += (size_t)blockIdx.y << logN;
   constexpr int KP = kPassMaxStages, K1 = KP / 2, K2 = KP - K1, G = kPassCols;
   constexpr int BW = (1 << K2) + 1, RW = (1 << K1) * BW;
   constexpr int NT1 = G << K2, NT2 = G << K1;
@@ -594,7 +641,12 @@ __device__ __forceinline__ void decode_row(int r, int D, int &e4, int &e3) {
 
 // residue of every output coefficient, times N^-1, in transform order: one warp per row (e4, e3), lanes over e2,
 // so the reads of the transform and the writes of the residues are contiguous
-__global__ void gather_kernel(const uint32_t *a, int D, int B, uint32_t ninv, uint32_t *res, PrimeQ P) {
+__global__ void gather_kernel(const uint32_t *a, int logN, int D, int B, int n_out, uint32_t *res,
+                              const __grid_constant__ Primes Q) {
+  const PrimeQ P = Q.P[blockIdx.y];
+  const uint32_t ninv = Q.ninv[blockIdx.y];
+  a += (size_t)blockIdx.y << logN;
+  res += (size_t)blockIdx.y * n_out;
   const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= tri(D + 1)) return;
   int e4, e3;
@@ -662,7 +714,7 @@ constexpr uint32_t kRoot[kPolyPowMaxPrimes] = {3u, 5u, 31u, 13u, 29u, 3u, 10u};
 static_assert(kQ[0] < 2ull * kQ[kPolyPowMaxPrimes - 1], "a residue mod an earlier prime reduces mod a later one by one subtraction");
 static_assert(kPolyPowLimbs == 8, "a coefficient record is two 16-byte stores");
 
-uint64_t host_mulmod(uint64_t a, uint64_t b, uint64_t q) { return (uint64_t)((unsigned __int128)a * b % q); }
+uint64_t host_mulmod(uint64_t a, uint64_t b, uint64_t q) { return a * b % q; }   // a, b < 2^32
 uint64_t host_powmod(uint64_t a, uint64_t e, uint64_t q) {
   uint64_t r = 1;
   a %= q;
@@ -719,11 +771,20 @@ int polypow_primes(uint64_t sum, int n) {
 // its companion.
 constexpr size_t kTwWords = 2 * (4096 + 4096 + kPassR / 2);
 
+// Primes whose transforms run side by side in one launch.  A transform of 2^20 words fills the device for a few
+// microseconds only, so small ones go together (n = 5, two primes: 18 launches and 124 us one after another); 64 MB of
+// them stay in L2 between the passes, which is where the line lies (n = 15: one prime of 64 MB at a time).
+int primes_at_once(uint32_t N, int nprimes) {
+  const uint32_t fit = (64u << 20) / 4u / N;
+  return fit < 1 ? 1 : fit < (uint32_t)nprimes ? (int)fit : nprimes;
+}
+
 size_t polypow_scratch_words(int d, int n, int nprimes) {
   const int B = d * n + 1;
   uint32_t N = 1;
   while ((uint64_t)N < (uint64_t)B * B * B) N <<= 1;
-  return (size_t)N + 2 * kTwWords * (size_t)nprimes + (size_t)nprimes * tet(d * n + 1) + tet(d + 1) + 64;
+  return (size_t)primes_at_once(N, nprimes) * N + 2 * kTwWords * (size_t)nprimes + (size_t)nprimes * tet(d * n + 1) +
+         tet(d + 1) + 64;
 }
 
 // Rows of the first forward column pass (kp0 stages; 0: no column pass) that can hold input, and the words cleared
@@ -786,14 +847,13 @@ TwTab plan_tables(uint32_t *tab, uint32_t w, uint32_t N, const PrimeQ &P, TableJ
   return T;
 }
 
-// One column pass of kp stages: the register-phase kernel for kp >= 2, the shared-memory stage loop for kp = 1.
-// nz_rows: rows of every column the forward pass reads (the rest are zero); the stage loop reads them all.
-void column_pass(bool inv, int kp, uint32_t blocks, uint32_t *a, int logN, int logM, const TwTab &T, const PrimeQ &P,
-                 cudaStream_t st, int nz_rows) {
-#define QFS_COLUMN_PASS(KP)                                                                               \
-  case KP:                                                                                                \
-    if (inv) ntt_column_regs<KP, true><<<blocks, kNttThreads, 0, st>>>(a, logN, logM, T, T, P, 1 << KP);  \
-    else ntt_column_regs<KP, false><<<blocks, kNttThreads, 0, st>>>(a, logN, logM, T, T, P, nz_rows);     \
+// One column pass of kp stages over `count` primes: the register-phase kernel for kp >= 2, the shared-memory stage loop
+// for kp = 1.  nz_rows: rows of every column the forward pass reads (the rest are zero); the stage loop reads them all.
+template <bool INV, bool ONE>
+void column_pass_of(int kp, dim3 grid, uint32_t *a, int logN, int logM, const Primes &Q, cudaStream_t st, int nz_rows) {
+#define QFS_COLUMN_PASS(KP)                                                                                           \
+  case KP:                                                                                                            \
+    ntt_column_regs<KP, INV, ONE><<<grid, kNttThreads, 0, st>>>(a, logN, logM, Q, INV ? 1 << KP : nz_rows);           \
     break;
   switch (kp) {
     QFS_COLUMN_PASS(2)
@@ -803,16 +863,20 @@ void column_pass(bool inv, int kp, uint32_t blocks, uint32_t *a, int logN, int l
     QFS_COLUMN_PASS(6)
     QFS_COLUMN_PASS(7)
     QFS_COLUMN_PASS(8)
-    default:
-      if (inv) ntt_column_pass<true><<<blocks, 256, 0, st>>>(a, logN, logM, kp, T, T, P);
-      else ntt_column_pass<false><<<blocks, 256, 0, st>>>(a, logN, logM, kp, T, T, P);
+    default: ntt_column_pass<INV><<<grid, 256, 0, st>>>(a, logN, logM, kp, Q);
   }
 #undef QFS_COLUMN_PASS
+}
+template <bool INV>
+void column_pass(int kp, uint32_t blocks, uint32_t *a, int logN, int logM, const Primes &Q, int count,
+                 cudaStream_t st, int nz_rows = 0) {
+  if (count == 1) column_pass_of<INV, true>(kp, dim3(blocks, 1), a, logN, logM, Q, st, nz_rows);
+  else column_pass_of<INV, false>(kp, dim3(blocks, count), a, logN, logM, Q, st, nz_rows);
 }
 
 }  // namespace
 
-cudaError_t polypow_launch(int d, int n, int nprimes, const uint32_t *coeffs_dev, uint32_t *out, uint32_t *scratch,
+cudaError_t polypow_launch(int d, int n, int nprimes, const uint32_t *coeffs, uint32_t *out, uint32_t *scratch,
                            cudaStream_t st) {
   const int B = d * n + 1, D = d * n;
   uint32_t N = 1;
@@ -820,9 +884,10 @@ cudaError_t polypow_launch(int d, int n, int nprimes, const uint32_t *coeffs_dev
   while ((uint64_t)N < (uint64_t)B * B * B) { N <<= 1; ++logN; }
   const int n_out = tet(D + 1);
   uint32_t *a = scratch;
-  uint32_t *tw = a + N;                               // forward and inverse tables of every prime
+  const int group = primes_at_once(N, nprimes);       // transforms side by side
+  uint32_t *tw = a + (size_t)group * N;               // forward and inverse tables of every prime
   uint32_t *res = tw + 2 * kTwWords * (size_t)nprimes;
-  const int grid = 152 * 8, block = 256;
+  const int block = 256;
   // passes: the innermost takes min(8, logN) stages on contiguous runs; the rest, outermost first, up to 8 each
   const int inner = logN < kPassMaxStages ? logN : kPassMaxStages;
   int outer[4], n_outer = 0;
@@ -833,9 +898,7 @@ cudaError_t polypow_launch(int d, int n, int nprimes, const uint32_t *coeffs_dev
   }
   CrtParams C;
   C.nprimes = nprimes;
-  PrimeQ PQ[kPolyPowMaxPrimes];
-  TwTab TF[kPolyPowMaxPrimes], TI[kPolyPowMaxPrimes];
-  uint32_t ninv[kPolyPowMaxPrimes];
+  Primes Q{};
   TableJobs J;
   int njobs = 0;
   for (int j = 0; j < nprimes; ++j) {
@@ -843,43 +906,59 @@ cudaError_t polypow_launch(int d, int n, int nprimes, const uint32_t *coeffs_dev
     uint32_t qinv = 1;   // q^-1 mod 2^32 by Newton's iteration (each step doubles the correct low bits)
     for (int i = 0; i < 5; ++i) qinv *= 2u - q * qinv;
     const uint32_t rmod = (uint32_t)((((uint64_t)1) << 32) % q);
-    PQ[j] = PrimeQ{q, barrett_mu(q), 0u - qinv, rmod, (uint32_t)host_mulmod(rmod, rmod, q)};
+    Q.P[j] = PrimeQ{q, barrett_mu(q), 0u - qinv, rmod, (uint32_t)host_mulmod(rmod, rmod, q)};
     C.q[j] = q;
-    C.mu[j] = PQ[j].mu;
+    C.mu[j] = Q.P[j].mu;
     for (int k = 0; k < kPolyPowMaxPrimes; ++k) C.inv[j][k] = k < j ? (uint32_t)host_powmod(kQ[k] % q, q - 2, q) : 0u;
     const uint32_t w = (uint32_t)host_powmod(kRoot[j], (q - 1) / N, q);   // primitive N-th root
     const uint32_t wi = (uint32_t)host_powmod(w, q - 2, q);
-    ninv[j] = (uint32_t)host_powmod(N, q - 2, q);
-    TF[j] = plan_tables(tw + 2 * kTwWords * (size_t)j, w, N, PQ[j], J, njobs);
-    TI[j] = plan_tables(tw + 2 * kTwWords * (size_t)j + kTwWords, wi, N, PQ[j], J, njobs);
+    Q.ninv[j] = (uint32_t)host_powmod(N, q - 2, q);
+    Q.cn[j] = (uint32_t)host_powmod(2, 32 * (uint64_t)n, q);
+    Q.F[j] = plan_tables(tw + 2 * kTwWords * (size_t)j, w, N, Q.P[j], J, njobs);
+    Q.I[j] = plan_tables(tw + 2 * kTwWords * (size_t)j + kTwWords, wi, N, Q.P[j], J, njobs);
   }
   power_tables_kernel<<<dim3(16, njobs), block, 0, st>>>(J);
   // the packed input occupies indices < d B^2 + 1, so the first forward pass (columns of stride N >> outer[0]) finds
   // it in its leading rows only: those rows are cleared and read, the others are zero without a read
   const PassRows PR = first_pass_rows(d, B, logN, n_outer ? outer[0] : 0);
-  for (int j = 0; j < nprimes; ++j) {
-    const PrimeQ &P = PQ[j];
-    zero_kernel<<<grid, block, 0, st>>>(a, PR.cleared);
-    scatter_kernel<<<64, block, 0, st>>>(coeffs_dev, d, B, a, P);
+  // inputs of up to kGivenCoeffs coefficients travel with the launches, larger ones through the scratch
+  const int n_in = tet(d + 1);
+  GivenCoeffs given;
+  const uint32_t *coeffs_dev = nullptr;
+  if (n_in <= kGivenCoeffs) {
+    for (int i = 0; i < n_in; ++i) given.c[i] = coeffs[i];
+  } else {
+    uint32_t *dev = res + (size_t)nprimes * n_out;
+    const cudaError_t e = cudaMemcpyAsync(dev, coeffs, sizeof(uint32_t) * n_in, cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return e;
+    coeffs_dev = dev;
+  }
+  for (int j = 0; j < nprimes; j += group) {
+    const int count = nprimes - j < group ? nprimes - j : group;
+    const Primes G = Q.from(j);
+    const uint32_t runs = (PR.cleared + B - 1) / B;
+    fill_kernel<<<dim3(runs / 8 + 1 < 1216 ? runs / 8 + 1 : 1216, count), block, 0, st>>>(given, coeffs_dev, d, B,
+                                                                                        PR.cleared, N, a, G);
     // forward: outer passes on blocks of M = N, N / 2^kp0, ...; the inner pass fuses the powers and the inverse
     int logM = logN;
     for (int i = 0; i < n_outer; ++i) {
-      column_pass(false, outer[i], (N >> outer[i]) / kPassCols, a, logN, logM, TF[j], P, st,
-                  i == 0 ? PR.rows : 1 << outer[i]);
+      column_pass<false>(outer[i], (N >> outer[i]) / kPassCols, a, logN, logM, G, count, st,
+                         i == 0 ? PR.rows : 1 << outer[i]);
       logM -= outer[i];
     }
     if (inner == kPassMaxStages && N >= (uint32_t)(kPassR * kPassCols)) {
-      const uint32_t cn = (uint32_t)host_powmod(2, 32 * (uint64_t)n, P.q);
-      ntt_inner_regs<<<N / (kPassR * kPassCols), kNttThreads, 0, st>>>(a, logN, (uint32_t)n, cn, TF[j], TI[j], P);
+      const dim3 grid(N / (kPassR * kPassCols), count);
+      if (count == 1) ntt_inner_regs<true><<<grid, kNttThreads, 0, st>>>(a, logN, (uint32_t)n, G);
+      else ntt_inner_regs<false><<<grid, kNttThreads, 0, st>>>(a, logN, (uint32_t)n, G);
     } else {
       const uint32_t inner_words = N < (uint32_t)(kPassR * kPassCols) ? N : (uint32_t)(kPassR * kPassCols);
-      ntt_inner_pow<<<N / inner_words, block, 0, st>>>(a, logN, inner, (uint32_t)n, TF[j], TI[j], P);
+      ntt_inner_pow<<<dim3(N / inner_words, count), block, 0, st>>>(a, logN, inner, (uint32_t)n, G);
     }
     for (int i = n_outer - 1; i >= 0; --i) {
       logM += outer[i];
-      column_pass(true, outer[i], (N >> outer[i]) / kPassCols, a, logN, logM, TI[j], P, st, 1 << outer[i]);
+      column_pass<true>(outer[i], (N >> outer[i]) / kPassCols, a, logN, logM, G, count, st);
     }
-    gather_kernel<<<(tri(D + 1) + 7) / 8, block, 0, st>>>(a, D, B, ninv[j], res + (size_t)j * n_out, P);
+    gather_kernel<<<dim3((tri(D + 1) + 7) / 8, count), block, 0, st>>>(a, logN, D, B, n_out, res + (size_t)j * n_out, G);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
