@@ -30,7 +30,8 @@ struct DeviceState {
   size_t total_mem = 0;
   void *ws = nullptr;          // persistent-CTA workspaces
   size_t ws_bytes = 0;
-  void *ctrl = nullptr;        // [0]: work counter (u64), [8]: status (u32), [16]: stats (2 x u64), [32]: survivors (u64)
+  void *ctrl = nullptr;        // [8]: status (u32), [16]: stats (2 x u64); cleared by every fused launch: [32]: survivors,
+                               // [40]: work counter (u64 each)
   void *staged = nullptr;      // staged-engine survivor buffers
   size_t staged_bytes = 0;
   int *which = nullptr;        // theta-matrix export: which workspace buffer holds each quartic's Delta
@@ -220,17 +221,49 @@ cudaError_t form_debug(int form, int p, const uint8_t *f, int max_h, int8_t *h_o
   }
 }
 
+cudaError_t form_crews(int form, int *active, int crew, size_t smem) {
+  return form == QFS_FORM_DP4A ? FormLauncher<1>::crews(active, crew, smem) : cudaErrorNotSupported;
+}
+
 bool form_supported(int form) { return form == QFS_FORM_INT32 || form == QFS_FORM_DP4A || form == QFS_FORM_INT8TC; }
 
 
+// Crews (clusters of CTAs per quartic, see qfs_common.cuh) of a dp4a chain launch at p >= 7.  One CTA per quartic is the
+// best use of the device while there are many; with few quartics past height 1, or with a few heavy ones (p = 11 beside
+// p = 5), CTAs run out of work while others are in the middle of a quartic.  A crew of 8 takes 0.56 ms for a quartic at
+// p = 7 that one CTA takes 2.2 ms for alone, but 300 quartics take 6.2 ms by crews of 8 and 4.4 ms by single CTAs, so the largest
+// crew that leaves every quartic one at once is taken (1,001 random quartics at p = 7: 6.1 -> 3.1 to 3.7 ms with the block
+// products, 5.4 ms without crews; 48 theta matrices: 3.1 -> 2.2 ms; p = 5, 7 and 11 together, 47 heavy quartics: 204 -> 83 ms).
+//   One prime: the number of survivors decides on the device.  A launch is made for each crew size that can come up,
+// and all but one find that it is not their turn.
+//   Several primes: estimated here from the share 1/p of quartics past height 1 and the outputs of their chains: the heaviest quartic
+// should take at most half of what the launch takes if its work is spread evenly.
+bool same_prime(const FusedParams &prm) {
+  for (int i = 1; i < prm.n_groups; ++i)
+    if (prm.g[i].p != prm.g[0].p) return false;
+  return true;
+}
+int mixed_crew(const FusedParams &prm, int slots) {
+  const double outputs[kMaxP + 1] = {0, 0, 0, 2e4, 0, 4.3e5, 0, 8.3e6, 0, 0, 0, 4e8, 0, 1.6e9};
+  double work = 0, heaviest = 0;
+  for (int i = 0; i < prm.n_groups; ++i) {
+    const int p = prm.g[i].p;
+    work += outputs[p] * std::max(1.0, (double)prm.g[i].n / p);
+    heaviest = std::max(heaviest, outputs[p]);
+  }
+  const double need = 2 * slots * heaviest / work;
+  return need >= 8 ? 8 : need >= 4 ? 4 : need >= 2 ? 2 : 1;
+}
+
 struct Plan {
-  int grid = 0;
+  int grid = 0;        // CTAs of a launch without crews
+  int crews[4] = {};   // crews of 2^i CTAs the device holds at once (0: not used)
   size_t smem = 0;
   size_t ws_words = 0;
 };
 
 int make_plan(DeviceState &S, int form, int max_p, int64_t n_items, const qfs_options_t *opts, Plan &plan,
-              size_t smem) {
+              size_t smem, const FusedParams *prm = nullptr) {
   plan.smem = smem;
   plan.ws_words = workspace_stride_words(max_p);
   int per_sm = opts && opts->ctas_per_sm > 0 ? opts->ctas_per_sm : 0;
@@ -248,10 +281,26 @@ int make_plan(DeviceState &S, int form, int max_p, int64_t n_items, const qfs_op
   const size_t per_cta = 2 * plan.ws_words * sizeof(uint32_t);
   const size_t budget = opts && opts->workspace_budget ? opts->workspace_budget : default_budget(S);
   grid = std::min<int64_t>(grid, (int64_t)(budget / per_cta));
+  int64_t ctas = std::min<int64_t>(grid, n_items);   // CTAs that need buffers
+  if (prm && max_p >= 7 && !(opts && (opts->ctas_per_sm > 0 || opts->max_ctas > 0))) {
+    const bool one_prime = same_prime(*prm);
+    const int want = one_prime ? 0 : mixed_crew(*prm, (int)grid);
+    // a batch of one prime with many rows will not leave few survivors
+    const bool few = one_prime && n_items / max_p <= 2 * grid;
+    for (int i = 1; i < 4; ++i) {
+      const int crew = 1 << i;
+      if (one_prime ? !few : crew != want) continue;
+      int active = 0;
+      const cudaError_t e = form_crews(form, &active, crew, smem);
+      if (e != cudaSuccess) return cuda_fail(e);
+      plan.crews[i] = (int)std::min<int64_t>({(int64_t)active, grid / crew, n_items});
+      ctas = std::max<int64_t>(ctas, (int64_t)plan.crews[i] * crew);
+    }
+  }
   grid = std::min<int64_t>(grid, n_items);
   if (grid < 1) return QFS_ERR_NO_MEMORY;
   plan.grid = (int)grid;
-  return ensure_workspace(S, workspace_words(grid, plan.ws_words) * sizeof(uint32_t));
+  return ensure_workspace(S, workspace_words(ctas, plan.ws_words) * sizeof(uint32_t));
 }
 
 }  // namespace
@@ -350,9 +399,12 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
                                                      uses_ring_chain(form, prm.g[i].p), power));
   const size_t smem = ring_offset_for(tet(4 * (max_p - 1) + 1)) + 4 * (size_t)ring_words;
   Plan plan;
-  rc = make_plan(*S, form, max_p, n_items, opts, plan, smem);
+  const bool one_prime = same_prime(prm);
+  rc = make_plan(*S, form, max_p, n_items, opts, plan, smem,
+                 form == QFS_FORM_DP4A && power == QFS_POWER_CHAIN ? &prm : nullptr);
   if (rc) return rc;
-  prm.counter = reinterpret_cast<unsigned long long *>(S->ctrl);
+  auto *n_list = reinterpret_cast<unsigned long long *>(static_cast<char *>(S->ctrl) + 32);
+  prm.counter = n_list + 1;
   prm.status = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(S->ctrl) + 8);
   prm.stats = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(S->ctrl) + 16);
   prm.ws = reinterpret_cast<uint32_t *>(S->ws);
@@ -360,18 +412,27 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
   // height-1 screen first: the persistent launch then runs only the quartics that pass it
   rc = ensure_list(*S, (size_t)n_items * sizeof(int64_t));
   if (rc) return rc;
-  auto *n_list = reinterpret_cast<unsigned long long *>(static_cast<char *>(S->ctrl) + 32);
-  cudaError_t e = cudaMemsetAsync(n_list, 0, sizeof(unsigned long long), stream);
+  cudaError_t e = cudaMemsetAsync(n_list, 0, 2 * sizeof(unsigned long long), stream);
   if (e != cudaSuccess) return cuda_fail(e);
   const int64_t screen_ctas = std::min<int64_t>((n_items + 7) / 8, (int64_t)S->sms * 8);
   e = screen_launch(prm, max_p, static_cast<int64_t *>(S->list), n_list, (int)screen_ctas, stream);
   if (e != cudaSuccess) return cuda_fail(e);
   prm.list = static_cast<const int64_t *>(S->list);
   prm.n_list = n_list;
-  e = cudaMemsetAsync(prm.counter, 0, sizeof(unsigned long long), stream);
-  if (e != cudaSuccess) return cuda_fail(e);
-  e = form_fused(form, prm, plan.grid, plan.smem, stream, form == QFS_FORM_INT8TC && max_p <= 5);
-  if (e != cudaSuccess) return cuda_fail(e);
+  int crews_at_once = 0;   // of the larger crews: up to so many survivors are theirs
+  for (int i = 3; i >= 0; --i) {
+    const int at_once = i > 0 ? plan.crews[i] : plan.grid;
+    if (at_once == 0) continue;
+    const bool last = i == 0 || !one_prime;   // several primes: one crew size, whatever the number of survivors
+    prm.crew = 1 << i;
+    prm.run_min = crews_at_once + 1;
+    prm.run_max = last ? INT64_MAX : at_once;
+    if (prm.run_min > n_items || prm.run_max < prm.run_min) continue;
+    e = form_fused(form, prm, i > 0 ? at_once << i : at_once, plan.smem, stream, form == QFS_FORM_INT8TC && max_p <= 5);
+    if (e != cudaSuccess) return cuda_fail(e);
+    if (last) break;
+    crews_at_once = at_once;
+  }
   return QFS_OK;
 }
 
@@ -398,6 +459,17 @@ int qfs_plan_prepare(int p, int64_t n_hint) {
   int64_t n = n_hint > 0 ? n_hint : (int64_t)1 << 40;
   for (int form : {QFS_FORM_INT32, QFS_FORM_DP4A, QFS_FORM_INT8TC}) {
     rc = make_plan(*S, form, p, n, nullptr, plan, smem_bytes_for(p, tile_for(p), uses_ring_chain(form, p)));
+    if (rc) return rc;
+  }
+  {   // the dp4a chain's own launches, crews included
+    FusedParams prm;
+    std::memset(&prm, 0, sizeof(prm));
+    prm.n_groups = 1;
+    prm.g[0].p = p;
+    prm.g[0].n = n;
+    const size_t smem = ring_offset_for(tet(4 * (p - 1) + 1)) +
+                        4 * (size_t)ring_words_for(p, tile_for(p), uses_ring_chain(QFS_FORM_DP4A, p), QFS_POWER_CHAIN);
+    rc = make_plan(*S, QFS_FORM_DP4A, p, n, nullptr, plan, smem, &prm);
     if (rc) return rc;
   }
   if (n_hint > 0) {
@@ -723,9 +795,13 @@ extern "C" int qfs_theta_matrix(int p, int64_t n, const uint8_t *coeffs, uint8_t
   const size_t ld = (size_t)tet(4 * (p - 1) + 1);
   // quartics per batch: one CTA each, bounded by the SM count and by the workspace budget
   int64_t batch = std::min<int64_t>(n, 2 * (int64_t)S->sms);
-  batch = std::min<int64_t>(batch, (int64_t)(default_budget(*S) / (2 * stride * sizeof(uint32_t))));
+  const int64_t fit = (int64_t)(default_budget(*S) / (2 * stride * sizeof(uint32_t)));
+  batch = std::min<int64_t>(batch, fit);
   if (batch < 1) return QFS_ERR_NO_MEMORY;
-  rc = ensure_workspace(*S, workspace_words(batch, stride) * sizeof(uint32_t));
+  // few quartics: a crew of CTAs for each (p >= 7), as many as the device holds at once
+  int crew = 1;
+  while (p >= 7 && crew < 8 && 2 * crew * batch <= std::min<int64_t>(2 * (int64_t)S->sms, fit)) crew *= 2;
+  rc = ensure_workspace(*S, workspace_words(batch * crew, stride) * sizeof(uint32_t));
   if (rc) return rc;
   if (S->which_n < batch) {
     if (S->which) cudaFree(S->which);
@@ -740,7 +816,7 @@ extern "C" int qfs_theta_matrix(int p, int64_t n, const uint8_t *coeffs, uint8_t
   uint32_t *status = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(S->ctrl) + 8);
   for (int64_t i0 = 0; i0 < n; i0 += batch) {
     const int nb = (int)std::min<int64_t>(batch, n - i0);
-    cudaError_t e = theta_matrix_launch(p, coeffs + 35 * i0, nb, M_out + (size_t)i0 * ld * ld,
+    cudaError_t e = theta_matrix_launch(p, coeffs + 35 * i0, nb, crew, M_out + (size_t)i0 * ld * ld,
                                         static_cast<uint32_t *>(S->ws), stride, S->which, status, stream);
     if (e != cudaSuccess) return cuda_fail(e);
   }

@@ -298,14 +298,16 @@ template <int P, bool LAST, bool DEBUG>
 __device__ __noinline__ void run_strips(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, int m_in,
                                         Smem &sm, uint32_t *ring, const uint8_t *gs, uint32_t *status,
                                         DebugPtrs dbg) {
-  constexpr int kTeam = team_threads(P), kTeams = kThreads / kTeam, kPerSlice = kTeam / kSlices;
+  constexpr int kTeam = team_threads(P), kOwn = kThreads / kTeam, kPerSlice = kTeam / kSlices;
   constexpr int kCopies = (Ring<P>::stride / 4 - 1 + kPerSlice - 1) / kPerSlice;   // 16-byte copies per thread and group
   const int m_out = m_in + 4;
   const int n_items = half_prefix(m_out + 1), n_strips = (n_items + kTeam - 1) / kTeam;
   const int team = (int)threadIdx.x / kTeam, tt = (int)threadIdx.x % kTeam;
   const int fs = tt / kPerSlice, fk = tt % kPerSlice;   // slice of a group and first chunk this thread copies
   ring += team * Ring<P>::words;
-  const int lg = unit_log2(m_out), seg = 1 << lg;   // blocks of a unit
+  // teams of the crew; a crew's units are shorter, so that there are enough of them
+  const int kTeams = kOwn * sm.crew, me = kOwn * sm.rank + team;
+  const int lg = max(1, unit_log2(m_out) - (sm.crew > 1 ? high_bit((unsigned)sm.crew) : 0)), seg = 1 << lg;   // blocks of a unit
   Taps T;
 #pragma unroll
   for (int uI = 1; uI < 5; ++uI) {
@@ -319,10 +321,19 @@ __device__ __noinline__ void run_strips(const uint32_t *__restrict__ in, uint32_
   // the zero chunk before each staged slice
   if (tt < kGroups * kSlices) *reinterpret_cast<uint4 *>(ring + tt * Ring<P>::stride) = make_uint4(0u, 0u, 0u, 0u);
 
-  // Unit queue of the product (counter (m_in / 4) mod 2; the other one is cleared for the next product).  Units are
-  // numbered strip after strip; a team's first two are fixed, the others come from the counter.
+  // Unit queue of the product (counter (m_in / 4) mod 2 of the crew's first CTA; the other one is cleared for the next
+  // product).  Units are numbered strip after strip; a team's first two are fixed, the others come from the counter.
   const int par = (m_in >> 2) & 1;
   if (threadIdx.x == 0) sm.unit_next[par ^ 1] = 0;
+  auto claim = [&]() {
+    if (sm.crew == 1) return atomicAdd(&sm.unit_next[par], 1);
+    int n;
+    asm volatile("atom.relaxed.cluster.shared::cluster.add.s32 %0, [%1], 1;"
+                 : "=r"(n)
+                 : "r"(crew_addr(&sm.unit_next[par], 0))
+                 : "memory");
+    return n;
+  };
   int cur_k = 0, cur_base = 0;   // cursor: strip and the number of units before it
   auto find = [&](int u) {       // unit u >= the last one -> strip | segment << 16, or -1 past the end
     while (cur_k < n_strips) {
@@ -335,7 +346,7 @@ __device__ __noinline__ void run_strips(const uint32_t *__restrict__ in, uint32_
     return -1;
   };
   // the unit being staged
-  int fid = find(team), f_g = 0, f_ng = 0, f_v = 0, f_hi = 0, f_base = 0, f_n = 0;
+  int fid = find(me), f_g = 0, f_ng = 0, f_v = 0, f_hi = 0, f_base = 0, f_n = 0;
   auto stage_unit = [&]() {
     if (fid < 0) { f_ng = 0; return; }
     const Strip S = strip_at(sm, fid & 0xFFFF, m_out);
@@ -350,7 +361,7 @@ __device__ __noinline__ void run_strips(const uint32_t *__restrict__ in, uint32_
   stage_unit();
   int uid = fid;                     // the unit being multiplied
   int q0 = -1, q1 = -1;              // units staged after it
-  int nxt = team + kTeams;           // the unit to stage after fid
+  int nxt = me + kTeams;             // the unit to stage after fid
   int qp = 0;
   bool want = false;
   // next group -> ring slot `slot`
@@ -364,7 +375,7 @@ __device__ __noinline__ void run_strips(const uint32_t *__restrict__ in, uint32_
       stage_unit();
       if (q0 < 0) q0 = fid; else q1 = fid;
       want = fid >= 0;
-      if (want && tt == 0) sm.unit_slot[team][qp] = 2 * kTeams + atomicAdd(&sm.unit_next[par], 1);
+      if (want && tt == 0) sm.unit_slot[team][qp] = 2 * kTeams + claim();
     }
     if (f_ng > 0) {
       const int v = f_v + fs;
@@ -447,8 +458,8 @@ __host__ __device__ constexpr int block_ring_words(int p) {
   return kThreads / block::team_threads(p) * block::kGroups * block::kSlices * block::slice_stride(p);
 }
 
-// The dp4a product (every tap pair, whatever sm.dense_min).  The caller runs it with every thread of the CTA, between
-// two barriers, after setup_quartic; consecutive products have degrees four apart or start again at degree 4 (their
+// The dp4a product (every tap pair, whatever sm.dense_min).  The caller runs it with every thread of the crew, between
+// two barriers of the crew, after setup_quartic; consecutive products have degrees four apart or start again at degree 4 (their
 // unit counters alternate); ring: block_ring_words words, 16-byte aligned.
 template <int P, bool LAST, bool DEBUG>
 __device__ __forceinline__ void block_chain_step(const uint32_t *__restrict__ in, uint32_t *__restrict__ out,

@@ -43,6 +43,37 @@ struct DebugPtrs {
   int32_t *iters;     // packed, (max_h-1) x ld
 };
 
+// Crews.  A launch over few quartics runs as thread-block clusters: the CTAs of a cluster (a crew, 1, 2, 4 or 8 of them)
+// work on one quartic together.  Each forms f^(p-1) for itself; the products of A4 and the theta steps are split, with
+// the forms in the first CTA's buffers.  Every CTA of a crew takes the same decisions from the same data.
+#if defined(__CUDACC__)
+__device__ __forceinline__ int crew_rank() {
+  unsigned r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return (int)r;
+}
+__device__ __forceinline__ int crew_size() {
+  unsigned n;
+  asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n));
+  return (int)n;
+}
+// Barrier over the crew; writes before it, to shared and global memory, are visible to the whole crew after it.
+__device__ __forceinline__ void crew_sync(int crew) {
+  if (crew > 1) {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  } else {
+    __syncthreads();
+  }
+}
+// The shared-memory address of a variable of this CTA in the CTA of the given rank.
+__device__ __forceinline__ uint32_t crew_addr(const void *p, int rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return a;
+}
+#endif
+
 struct Smem {
   int SW[kSWLen];
   int taps[35];           // coefficients of f, packed order (index tet(uI) + tri(sI) + tI)
@@ -63,6 +94,7 @@ struct Smem {
   int64_t item;
   int flag;
   int task_next;   // swept chain: next task of the current product (work queue shared by the CTA's warps)
+  int crew, rank;  // CTAs working on this quartic's products together, and this one's place (1 and 0: alone)
   int task_done;   // swept chain: warps that found the queue empty; the last one resets both counters
   // followed in dynamic shared memory by two byte arrays of ld entries: g (current iterate) and g_next
 };

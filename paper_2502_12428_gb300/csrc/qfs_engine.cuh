@@ -630,18 +630,18 @@ __host__ __device__ inline int theta_ring_words_for(int p, int power) {
 
 // Padded Delta (degree D) -> guarded copy.  One thread per 16-byte chunk; the thread of a column's first chunk
 // writes the guard before the column, the thread of a slice's last chunk the guard after it.  The caller
-// synchronises the CTA afterwards.
+// synchronises the crew afterwards.
 template <int P>
 __device__ __forceinline__ void delta_to_guarded(const uint32_t *__restrict__ delta, uint32_t *__restrict__ dg,
                                                  const Smem &sm) {
   constexpr int D = Prime<P>::D;
   const int nchunks = sm.SW[D + 1] / 4;
   const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-  for (int k = threadIdx.x; k < nchunks; k += blockDim.x) {
+  for (int k = threadIdx.x + blockDim.x * sm.rank; k < nchunks; k += blockDim.x * sm.crew) {
     int u, s, c;
     decode_form_chunk(k, D, sm.SW, u, s, c);
     const int o = sm.SW[u] + theta_gsw_extra(u) + kThetaGuardWords * (s + 1) + colw(s) + 4 * c;
-    *reinterpret_cast<uint4 *>(dg + o) = *reinterpret_cast<const uint4 *>(delta + 4 * k);
+    *reinterpret_cast<uint4 *>(dg + o) = __ldcg(reinterpret_cast<const uint4 *>(delta + 4 * k));   // a crew's write
     if (c == 0)
 #pragma unroll
       for (int w = 0; w < kThetaGuardWords; w += 4) *reinterpret_cast<uint4 *>(dg + o - kThetaGuardWords + w) = z;
@@ -652,7 +652,7 @@ __device__ __forceinline__ void delta_to_guarded(const uint32_t *__restrict__ de
 }
 
 // One theta step: g (shared, packed) -> gn (shared, packed), Delta guarded in global memory.  One thread per
-// output; returns whether some output is nonzero (same value in every thread).
+// output, the outputs split over the crew; returns whether some output is nonzero (same value in every thread).
 template <int P>
 __device__ __noinline__ bool theta_gather(const uint32_t *__restrict__ dg, const Smem &sm,
                                           const uint8_t *__restrict__ g, uint8_t *__restrict__ gn, uint32_t *ring) {
@@ -684,7 +684,7 @@ __device__ __noinline__ bool theta_gather(const uint32_t *__restrict__ dg, const
   }
   __syncthreads();
   bool any = false;
-  for (int r = tid; r < Pr::ld; r += nthreads) {
+  for (int r = tid + nthreads * sm.rank; r < Pr::ld; r += nthreads * sm.crew) {
     int ur, sr, tr;
     decode_packed(r, ur, sr, tr, d);
     const int Ue = P * ur + 3 * (P - 1), Se = P * sr + 2 * (P - 1), Te = P * tr + (P - 1);
@@ -720,7 +720,15 @@ __device__ __noinline__ bool theta_gather(const uint32_t *__restrict__ dg, const
     }
     const int v = (int)(acc % P);
     gn[r] = (uint8_t)v;
+    for (int k = 1; k < sm.crew; ++k) {   // and into the other CTAs' gn
+      const int to = sm.rank + k < sm.crew ? sm.rank + k : sm.rank + k - sm.crew;
+      asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(crew_addr(gn + r, to)), "r"(v) : "memory");
+    }
     any |= v != 0;
+  }
+  if (sm.crew > 1) {
+    crew_sync(sm.crew);
+    for (int r = tid; r < Pr::ld; r += nthreads) any |= gn[r] != 0;
   }
   return __syncthreads_or(any ? 1 : 0) != 0;
 }
@@ -824,17 +832,19 @@ __device__ __noinline__ bool theta_stream(const uint32_t *__restrict__ delta, co
     const int n = chunk_prefix(eu + 1);
     for (int k = tid; k < n; k += nthreads) cp_async16(dst + ctab[k], src + 4 * k, true);
   };
-  // slices 0 .. NS-2 in flight; round e_u waits for its own slice, then refills the slot round e_u - 1 used
+  // the crew's CTAs take the slices in turns; slot i % NS holds this CTA's i-th slice: slices 0 .. NS-2 in flight, round i
+  // waits for its own slice, then refills the slot round i - 1 used
+  const int crew = sm.crew, rank = sm.rank;
   for (int e = 0; e < NS - 1; ++e) {
-    if (e <= D) fetch(e, e);
+    if (rank + e * crew <= D) fetch(rank + e * crew, e);
     cp_async_commit();
   }
-  for (int eu = 0; eu <= D; ++eu) {
+  for (int i = 0, eu = rank; eu <= D; ++i, eu += crew) {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(NS - 2));
-    __syncthreads();   // slot eu % NS is complete for every thread; slot (eu - 1) % NS is no longer read
-    if (eu + NS - 1 <= D) fetch(eu + NS - 1, (eu + NS - 1) % NS);
+    __syncthreads();   // slot i % NS is complete for every thread; slot (i - 1) % NS is no longer read
+    if (eu + (NS - 1) * crew <= D) fetch(eu + (NS - 1) * crew, (i + NS - 1) % NS);
     cp_async_commit();
-    const uint32_t *slot = slots + (eu % NS) * SLOT;
+    const uint32_t *slot = slots + (i % NS) * SLOT;
     // output slices with u_c = p u_r + 3(p-1) - e_u in [0, d]
     const int base = eu - 3 * (P - 1);
     const int ur_lo = max(0, (base + P - 1) / P);
@@ -885,13 +895,21 @@ __device__ __noinline__ bool theta_stream(const uint32_t *__restrict__ delta, co
     }
   }
   cp_async_wait_all();
-  __syncthreads();
+  crew_sync(crew);
   bool any = false;
   for (int r = tid; r < ld; r += nthreads) {
-    const int v = acc[r] % P;
+    int sum = acc[r];
+    for (int k = 1; k < crew; ++k) {   // the other CTAs' sums
+      const int from = rank + k < crew ? rank + k : rank + k - crew;
+      int x;
+      asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(x) : "r"(crew_addr(acc + r, from)) : "memory");
+      sum += x;
+    }
+    const int v = sum % P;
     gn[r] = (uint8_t)v;
     any |= v != 0;
   }
+  if (crew > 1) crew_sync(crew);   // nobody reads these sums any more
   return __syncthreads_or(any ? 1 : 0) != 0;
 }
 
@@ -977,7 +995,7 @@ __device__ __forceinline__ void delta_to_classes(const uint32_t *__restrict__ de
   for (int k = threadIdx.x; k < nchunks; k += blockDim.x) {
     int U, S, c;
     decode_form_chunk(k, D, sm.SW, U, S, c);
-    const uint4 v = *reinterpret_cast<const uint4 *>(delta + 4 * k);
+    const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(delta + 4 * k));   // a crew's write
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
     const int e2 = U - S, q2 = e2 / P, r2 = e2 - P * q2;
     const int T0 = 16 * c;
@@ -1209,12 +1227,12 @@ __device__ __forceinline__ void power_to_G(Smem &sm, const uint8_t *gs, uint32_t
   int m = Pr::d;
   for (int k = P - 1; k <= P * (P - 1) - 2; ++k) {
     chain_step<P, FORM, false, DEBUG>(cur, nxt, m, sm, ring, gs, status, dbg);
-    __syncthreads();
+    crew_sync(sm.crew);
     uint32_t *t = cur; cur = nxt; nxt = t;
     m += 4;
   }
   chain_step<P, FORM, LAST_DELTA, DEBUG>(cur, last_out ? last_out : nxt, m, sm, ring, gs, status, dbg);
-  __syncthreads();
+  crew_sync(sm.crew);
 }
 
 // The identity power mode at p <= 7, by residue classes: Delta_1(f^(p-1)) = E(x^p) - f^(p-2)(x^p) Delta_1(f) (mod p)
@@ -1577,11 +1595,12 @@ __device__ __noinline__ int reduced_height(Smem &sm, uint8_t *gs, uint8_t *gn, u
   return 0;
 }
 
-// Runs A1-A7 for one quartic with the CTA's two workspace buffers; returns the height code.
+// Runs A1-A7 for one quartic with the CTA's two workspace buffers; returns the height code.  crewA: the first of the
+// crew's buffers if the CTA belongs to one (chain power mode, dp4a form), else null.
 template <int P, int FORM, bool DEBUG>
 __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem &sm, uint8_t *gs, uint8_t *gn,
                                uint32_t *ring, uint32_t *bufA, uint32_t *bufB, uint32_t *status, DebugPtrs dbg,
-                               int &theta_steps, int power_mode = 0) {
+                               int &theta_steps, int power_mode = 0, uint32_t *crewA = nullptr) {
   using Pr = Prime<P>;
   const int tid = threadIdx.x;
   theta_steps = 0;
@@ -1591,6 +1610,22 @@ __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem 
   if (DEBUG)
     for (int i = tid; i < Pr::ld; i += blockDim.x) dbg.g[i] = gs[i];
   if (gs[Pr::witness] != 0) return 1;
+  uint32_t *own = bufA;   // a buffer that a crew leaves to this CTA, unless it is the first one
+  if constexpr (FORM == 1 && !DEBUG) {
+    // from here on the crew works in its first CTA's buffers
+    if (crewA) {
+      cur = cur == bufA ? crewA : crewA + (bufB - bufA);
+      other = other == bufA ? crewA : crewA + (bufB - bufA);
+      bufB = crewA + (bufB - bufA);
+      bufA = crewA;
+      if (tid == 0) {
+        sm.crew = crew_size();
+        sm.rank = crew_rank();
+      }
+      __syncthreads();
+      crew_sync(sm.crew);
+    }
+  }
   if (power_mode == 2)
     return reduced_height<P, FORM, DEBUG>(sm, gs, gn, ring, cur, other, max_h, status, dbg, theta_steps);
   // A4 + A5 into `other` or `cur`, whichever the chain's parity leaves last
@@ -1616,13 +1651,15 @@ __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem 
     if (in_classes) {
       dg = delta;
     } else if (by_classes) {
+      // (theta by classes is not split: each CTA of a crew makes its own copy, in its own order of classes)
+      if (sm.rank != 0) dg = own;
       poly_tables<P>(ringb);
       delta_to_classes<P>(delta, dg, sm, ringb);
     }
   } else {
     delta_to_guarded<P>(delta, dg, sm);
   }
-  __syncthreads();
+  crew_sync(sm.crew);
   uint8_t *g = gs, *g2 = gn;
   for (int h = 2; h <= max_h; ++h) {
     bool nonzero;
@@ -1667,6 +1704,8 @@ struct FusedParams {
   unsigned long long *stats;          // [0] quartics past the height-1 test, [1] theta steps run
   uint32_t *ws;                       // workspace: a guard, then 2 buffers of ws_words (the stride) per CTA
   size_t ws_words;
+  int crew;                           // CTAs per cluster of the launch (1: no clusters)
+  int64_t run_min, run_max;           // the launch does nothing unless the items to run are run_min .. run_max
   int power_mode;                     // 0: chain (Algorithm 1 literally), 1: identity shortcut, 2: reduced theta
   const int64_t *list;                // if set: the items to run (the survivors of the height-1 screen) ...
   const unsigned long long *n_list;   // ... and their count; if null, every item 0 .. n_items-1 runs
@@ -1677,6 +1716,8 @@ struct FusedParams {
 template <int FORM, bool SMALL>
 __device__ __forceinline__ void fused_body(const FusedParams &prm) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int64_t n_run = prm.list ? (int64_t)*prm.n_list : prm.n_items;
+  if (FORM == 1 && (n_run < prm.run_min || n_run > prm.run_max)) return;
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
   uint8_t *gs = smem_raw + sizeof(Smem);
   // the second iterate buffer follows the largest ld in this launch
@@ -1689,14 +1730,21 @@ __device__ __forceinline__ void fused_body(const FusedParams &prm) {
   uint32_t *bufA, *bufB;
   cta_buffers(prm.ws, prm.ws_words, bufA, bufB);
   DebugPtrs dbg{nullptr, nullptr, nullptr, nullptr};
-  const int64_t n_run = prm.list ? (int64_t)*prm.n_list : prm.n_items;
+  const int crew = FORM == 1 ? prm.crew : 1, rank = crew > 1 ? crew_rank() : 0;
+  uint32_t *crewA = crew > 1 ? bufA - (size_t)rank * 2 * prm.ws_words : nullptr;
   for (;;) {
-    __syncthreads();
+    crew_sync(crew);
     if (threadIdx.x == 0) {
-      const int64_t k = (int64_t)atomicAdd(prm.counter, 1ull);
-      sm.item = k < n_run ? (prm.list ? prm.list[k] : k) : -1;
+      sm.crew = 1;   // until f^(p-1) is formed
+      sm.rank = 0;
+      if (rank == 0) {
+        const int64_t k = (int64_t)atomicAdd(prm.counter, 1ull);
+        sm.item = k < n_run ? (prm.list ? prm.list[k] : k) : -1;
+        for (int to = 1; to < crew; ++to)
+          asm volatile("st.shared::cluster.s64 [%0], %1;" ::"r"(crew_addr(&sm.item, to)), "l"(sm.item) : "memory");
+      }
     }
-    __syncthreads();
+    crew_sync(crew);
     const int64_t item = sm.item;
     if (item < 0) break;
     int gi = 0;
@@ -1711,21 +1759,21 @@ __device__ __forceinline__ void fused_body(const FusedParams &prm) {
     const uint8_t *f = G.coeffs + 35 * row;
     int h, steps;
     switch (G.p) {
-      case 3: h = process_quartic<3, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode); break;
-      case 5: h = process_quartic<5, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode); break;
+      case 3: h = process_quartic<3, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA); break;
+      case 5: h = process_quartic<5, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA); break;
       default:
         if constexpr (SMALL) {
           h = -1;   // not reached: the host launches the small-prime kernel only when every group has p <= 5
         } else {
           switch (G.p) {
-            case 7: h = process_quartic<7, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode); break;
-            case 11: h = process_quartic<11, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode); break;
-            default: h = process_quartic<13, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode); break;
+            case 7: h = process_quartic<7, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA); break;
+            case 11: h = process_quartic<11, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA); break;
+            default: h = process_quartic<13, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA); break;
           }
         }
         break;
     }
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && rank == 0) {
       G.heights[row] = (int8_t)h;
       if (h != 1 && h != -1) {
         atomicAdd(prm.stats, 1ull);

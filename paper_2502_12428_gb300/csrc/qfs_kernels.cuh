@@ -1,6 +1,7 @@
 // Kernel entry points of one arithmetic form (instantiated once per form in its own translation unit).
 #pragma once
 #include <cuda_runtime.h>
+#include <utility>
 #include "qfs_engine.cuh"
 
 namespace qfs {
@@ -43,11 +44,46 @@ __global__ void __launch_bounds__(kThreads) debug_kernel(const uint8_t *f, int m
   if (threadIdx.x == 0) *h_out = (int8_t)h;
 }
 
+// A launch of `grid` CTAs in clusters of `crew` (1: none).
+template <typename... Params, typename... Args>
+cudaError_t launch_crews(void (*kernel)(Params...), int grid, int crew, size_t smem, cudaStream_t st, Args &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)crew;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = crew > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+// Clusters of `crew` CTAs that the device holds at once.
+template <typename... Params>
+cudaError_t active_crews(int *active, void (*kernel)(Params...), int crew, size_t smem) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)crew);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)crew;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaOccupancyMaxActiveClusters(active, kernel, &cfg);
+}
+
 // Host-side launchers (defined in qfs_form_<name>.cu).
 template <int FORM>
 struct FormLauncher {
   static cudaError_t fused(const FusedParams &prm, int grid, size_t smem, cudaStream_t st, bool small);
   static cudaError_t occupancy(int *blocks_per_sm, size_t smem, bool small);
+  static cudaError_t crews(int *active, int crew, size_t smem);   // clusters of `crew` CTAs the device holds at once
   static cudaError_t debug(int p, const uint8_t *f, int max_h, int8_t *h_out, uint32_t *bufA, uint32_t *bufB,
                            uint32_t *status, DebugPtrs dbg, cudaStream_t st, int power_mode);
 };
@@ -63,8 +99,7 @@ struct FormLauncher {
     auto k = small ? fused_kernel_small<FORM> : fused_kernel<FORM>;                                           \
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);          \
     if (e != cudaSuccess) return e;                                                                           \
-    k<<<grid, kThreads, smem, st>>>(prm);                                                                     \
-    return cudaGetLastError();                                                                                \
+    return launch_crews(k, grid, prm.crew, smem, st, prm);                                                    \
   }                                                                                                           \
   template <>                                                                                                 \
   cudaError_t FormLauncher<FORM>::occupancy(int *blocks_per_sm, size_t smem, bool small) {                    \
@@ -72,6 +107,10 @@ struct FormLauncher {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);          \
     if (e != cudaSuccess) return e;                                                                           \
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, kThreads, smem);                   \
+  }                                                                                                           \
+  template <>                                                                                                 \
+  cudaError_t FormLauncher<FORM>::crews(int *active, int crew, size_t smem) {                                 \
+    return active_crews(active, fused_kernel<FORM>, crew, smem);                                              \
   }
 
 #define QFS_DEFINE_DEBUG_LAUNCHER(FORM)                                                                       \

@@ -41,6 +41,8 @@ __device__ __forceinline__ void init_task_queue(Smem &sm) {
   if (threadIdx.x == 0) {
     sm.task_next = 0;
     sm.task_done = 0;
+    sm.crew = 1;
+    sm.rank = 0;
   }
 }
 

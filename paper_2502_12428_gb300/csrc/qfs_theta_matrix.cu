@@ -3,9 +3,9 @@
 // index p r + (p-1)1 - c falls outside the degree-D cone.  theta(g) = M g (mod p) for every form g of degree d.
 // The height pipeline never forms M (it produces theta(g) directly); this file exports it.
 //
-// Two kernels per batch of quartics: one CTA per quartic runs A1, A2, A4 and A5 unconditionally (the Fedder test
-// does not stop it) into the CTA's workspace buffers and records which buffer holds Delta; then a grid fills the
-// rows of every M from Delta.
+// Two kernels per batch of quartics: one crew (cluster) of CTAs per quartic runs A1, A2, A4 and A5 unconditionally (the
+// Fedder test does not stop it) into its first CTA's workspace buffers and records which buffer holds Delta; then a
+// grid fills the rows of every M from Delta.
 #include <cuda_runtime.h>
 
 #include "../../include/qfs.h"
@@ -16,7 +16,7 @@ namespace qfs {
 namespace {
 
 template <int P>
-__global__ void __launch_bounds__(kThreads, 1) theta_delta_kernel(const uint8_t *__restrict__ coeffs, uint32_t *ws,
+__global__ void __launch_bounds__(kThreads, 2) theta_delta_kernel(const uint8_t *__restrict__ coeffs, uint32_t *ws,
                                                                   size_t stride, int *which, uint32_t *status) {
   using Pr = Prime<P>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -34,16 +34,28 @@ __global__ void __launch_bounds__(kThreads, 1) theta_delta_kernel(const uint8_t 
   cta_buffers(ws, stride, bufA, bufB);
   __syncthreads();
   DebugPtrs dbg{nullptr, nullptr, nullptr, nullptr};
-  if (!setup_quartic<P>(coeffs + 35 * (size_t)blockIdx.x, sm)) {
-    if (threadIdx.x == 0) which[blockIdx.x] = -1;   // a coefficient >= p: M is left zero
+  const int crew = crew_size(), rank = crew_rank(), q = (int)blockIdx.x / crew;
+  if (!setup_quartic<P>(coeffs + 35 * (size_t)q, sm)) {   // the same for the whole crew
+    if (threadIdx.x == 0 && rank == 0) which[q] = -1;   // a coefficient >= p: M is left zero
     return;
   }
   uint32_t *cur = power_to_g<P, QFS_FORM_DP4A, false>(sm, gs, ring, bufA, bufB, status, dbg);
-  uint32_t *other = cur == bufA ? bufB : bufA;
+  // from here on the crew works in its first CTA's buffers
+  const bool in_a = cur == bufA;
+  bufA -= (size_t)rank * 2 * stride;
+  bufB = bufA + stride;
+  cur = in_a ? bufA : bufB;
+  uint32_t *other = in_a ? bufB : bufA;
+  if (threadIdx.x == 0) {
+    sm.crew = crew;
+    sm.rank = rank;
+  }
+  __syncthreads();
+  crew_sync(crew);
   constexpr int nsteps = P * (P - 1) - (P - 1);   // products from f~^(p-1) to f~^(p(p-1))
   uint32_t *delta = (nsteps % 2) ? other : cur;
   power_to_G<P, QFS_FORM_DP4A, true, false>(sm, gs, ring, cur, other, nullptr, status, dbg);
-  if (threadIdx.x == 0) which[blockIdx.x] = delta == bufA ? 0 : 1;
+  if (threadIdx.x == 0 && rank == 0) which[q] = delta == bufA ? 0 : 1;
 }
 
 // M rows [blockIdx.x * kRows, ...) of quartic blockIdx.y.  Dynamic shared memory: SW (D+2 ints) and the (u, s, t) of
@@ -51,8 +63,8 @@ __global__ void __launch_bounds__(kThreads, 1) theta_delta_kernel(const uint8_t 
 constexpr int kRows = 8;
 
 template <int P>
-__global__ void __launch_bounds__(kThreads) theta_matrix_fill(const uint32_t *ws, size_t stride, const int *which,
-                                                              uint8_t *M) {
+__global__ void __launch_bounds__(kThreads) theta_matrix_fill(const uint32_t *ws, size_t stride, int crew,
+                                                              const int *which, uint8_t *M) {
   using Pr = Prime<P>;
   constexpr int d = Pr::d, D = Pr::D, ld = Pr::ld;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -67,7 +79,7 @@ __global__ void __launch_bounds__(kThreads) theta_matrix_fill(const uint32_t *ws
   __syncthreads();
   const int q = blockIdx.y;
   const int w = which[q];
-  const uint8_t *delta = reinterpret_cast<const uint8_t *>(ws + kGuardWords + (2 * (size_t)q + (w > 0)) * stride);
+  const uint8_t *delta = reinterpret_cast<const uint8_t *>(ws + kGuardWords + (2 * (size_t)q * crew + (w > 0)) * stride);
   uint8_t *Mq = M + (size_t)q * ld * ld;
   const int r_end = min(ld, (int)(blockIdx.x + 1) * kRows);
   for (int r = blockIdx.x * kRows; r < r_end; ++r) {
@@ -87,32 +99,32 @@ __global__ void __launch_bounds__(kThreads) theta_matrix_fill(const uint32_t *ws
 }
 
 template <int P>
-cudaError_t launch(const uint8_t *coeffs, int n, uint8_t *M, uint32_t *ws, size_t stride, int *which,
+cudaError_t launch(const uint8_t *coeffs, int n, int crew, uint8_t *M, uint32_t *ws, size_t stride, int *which,
                    uint32_t *status, cudaStream_t st) {
   using Pr = Prime<P>;
   const size_t smem = smem_bytes_for(P, uses_ring_chain(QFS_FORM_DP4A, P));
   cudaError_t e = cudaFuncSetAttribute(theta_delta_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  theta_delta_kernel<P><<<n, kThreads, smem, st>>>(coeffs, ws, stride, which, status);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  e = launch_crews(theta_delta_kernel<P>, n * crew, crew, smem, st, coeffs, ws, stride, which, status);
+  if (e != cudaSuccess) return e;
   const size_t fsmem = sizeof(int) * (Pr::D + 2) + sizeof(uint32_t) * Pr::ld;
   e = cudaFuncSetAttribute(theta_matrix_fill<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem);
   if (e != cudaSuccess) return e;
   const dim3 grid((Pr::ld + kRows - 1) / kRows, n);
-  theta_matrix_fill<P><<<grid, kThreads, fsmem, st>>>(ws, stride, which, M);
+  theta_matrix_fill<P><<<grid, kThreads, fsmem, st>>>(ws, stride, crew, which, M);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t theta_matrix_launch(int p, const uint8_t *coeffs, int n, uint8_t *M, uint32_t *ws, size_t stride,
+cudaError_t theta_matrix_launch(int p, const uint8_t *coeffs, int n, int crew, uint8_t *M, uint32_t *ws, size_t stride,
                                 int *which, uint32_t *status, cudaStream_t st) {
   switch (p) {
-    case 3: return launch<3>(coeffs, n, M, ws, stride, which, status, st);
-    case 5: return launch<5>(coeffs, n, M, ws, stride, which, status, st);
-    case 7: return launch<7>(coeffs, n, M, ws, stride, which, status, st);
-    case 11: return launch<11>(coeffs, n, M, ws, stride, which, status, st);
-    default: return launch<13>(coeffs, n, M, ws, stride, which, status, st);
+    case 3: return launch<3>(coeffs, n, crew, M, ws, stride, which, status, st);
+    case 5: return launch<5>(coeffs, n, crew, M, ws, stride, which, status, st);
+    case 7: return launch<7>(coeffs, n, crew, M, ws, stride, which, status, st);
+    case 11: return launch<11>(coeffs, n, crew, M, ws, stride, which, status, st);
+    default: return launch<13>(coeffs, n, crew, M, ws, stride, which, status, st);
   }
 }
 

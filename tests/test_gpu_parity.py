@@ -212,6 +212,42 @@ def test_multi_group_with_empty_groups(qfs):
     assert all(o.numel() == 0 for o in outs)
 
 
+# ------------------------------------------------------------------------------------- crews of CTAs
+@pytest.mark.parametrize("p,n,pool", [(7, 1, 60), (7, 3, 60), (7, 40, 600), (11, 2, 60), (13, 1, 60)])
+def test_few_quartics_run_by_crews_of_ctas(qfs, p, n, pool):
+    # few quartics: clusters of CTAs split the products and the theta steps of each; every repetition splits
+    # them differently; the caps leave one CTA per quartic
+    f, h = find_rows(p, pool, 9700 + p, lambda x: x != 1, n)
+    assert len(f) == n
+    t = dev_tensor(f)
+    for kw in [{}] * (6 if p == 7 else 2) + [{"max_ctas": 1}, {"max_ctas": 5}, {"ctas_per_sm": 1}]:
+        if p == 13 and kw.get("max_ctas") == 1:
+            continue
+        assert np.array_equal(gpu_heights(qfs, p, f, **kw), h)
+    assert qfs.read_status() == 0
+    # a captured launch replays
+    out = torch.empty(n, dtype=torch.int8, device="cuda:0")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        qfs.heights(p, t, out=out)
+    for _ in range(2):
+        out.fill_(-5)
+        g.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(out.cpu().numpy(), h)
+
+
+def test_theta_matrix_by_crews_repeats(qfs):
+    f = dev_tensor(np.concatenate([inputs.dense(7, 3, 9800), inputs.sparse(7, 2, 9801)]))
+    ref = qfs.theta_matrix(7, f).cpu().numpy()
+    assert np.array_equal(ref[4], oracle.theta_matrix(7, f[4].cpu().numpy()))
+    for _ in range(4):
+        assert np.array_equal(qfs.theta_matrix(7, f).cpu().numpy(), ref)
+    assert np.array_equal(qfs.theta_matrix(7, f[:1]).cpu().numpy(), ref[:1])
+    assert qfs.read_status() == 0
+
+
 # ------------------------------------------------------------------------------------- edge cases and errors
 def test_edge_cases(qfs):
     p = 5
