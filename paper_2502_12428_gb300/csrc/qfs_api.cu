@@ -13,6 +13,7 @@
 #include "qfs_kernels.cuh"
 #include "qfs_matmul.cuh"
 #include "qfs_polypow.cuh"
+#include "qfs_reduced.cuh"
 #include "qfs_staged.cuh"
 #include "qfs_screen.cuh"
 #include "qfs_theta_matrix.cuh"
@@ -392,6 +393,13 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
   prm.power_mode = power;
   if (engine == QFS_ENGINE_STAGED) return run_staged(*S, prm, opts, stream);
 
+  // the reduced mode of one small prime (dp4a form) has a kernel of its own, which needs no workspace; a call that caps
+  // the CTAs or mixes primes takes the fused kernel
+  int reduced_p = 0;
+  if (power == QFS_POWER_REDUCED && form == QFS_FORM_DP4A && max_p <= kReducedMaxP &&
+      !(opts && (opts->ctas_per_sm > 0 || opts->max_ctas > 0))) {
+    reduced_p = same_prime(prm) ? max_p : 0;
+  }
   // shared memory: the largest iterate pair of the launch plus the largest ring any group's tile needs
   int ring_words = 0;
   for (int i = 0; i < prm.n_groups; ++i)
@@ -419,6 +427,7 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
   if (e != cudaSuccess) return cuda_fail(e);
   prm.list = static_cast<const int64_t *>(S->list);
   prm.n_list = n_list;
+  if (reduced_p) return (e = reduced_launch(reduced_p, prm, S->sms, stream)) == cudaSuccess ? QFS_OK : cuda_fail(e);
   int crews_at_once = 0;   // of the larger crews: up to so many survivors are theirs
   for (int i = 3; i >= 0; --i) {
     const int at_once = i > 0 ? plan.crews[i] : plan.grid;

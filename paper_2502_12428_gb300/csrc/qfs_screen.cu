@@ -5,11 +5,13 @@
 //
 // With k = (p-1)/2, f^(p-1) = F * F for F = f^k, so the coefficient is sum_a F[a] F[(p-1)1 - a] over the
 // monomials a of degree 2(p-1) whose four exponents are all <= p-1 (exactly the a for which (p-1)1 - a is a
-// monomial).  F is formed mod p by k-1 products with f in the warp's shared memory: in cone coordinates
-// (u, s, t) = (e2+e3+e4, e3+e4, e4) a product of forms is a 3-D convolution over the cone t <= s <= u <= degree.
+// monomial).  F is formed mod p by k-1 products with f in the warp's shared memory, by rows (qfs_rows.cuh): one output
+// word per lane, the taps by dp4a.  Bound by instruction issue.  262,144 quartics at p = 7 took 3.5 ms with
+// one output and 35 byte loads at a time, 0.74 ms this way.
 #include <cuda_runtime.h>
 
 #include "qfs_layout.cuh"
+#include "qfs_rows.cuh"
 #include "qfs_screen.cuh"
 
 namespace qfs {
@@ -17,61 +19,25 @@ namespace {
 
 constexpr int kScreenWarps = kScreenThreads / 32;
 
-// Bytes of one warp's region for primes up to max_p: f (35, padded to 48) and two buffers of C(4k+3, 3).
-__host__ __device__ constexpr int screen_buf_bytes(int max_p) {
-  return (tet(4 * ((max_p - 1) / 2) + 1) + 15) & ~15;
+// One warp's region for primes up to max_p, in words: the tap words, f (35 bytes), and two forms of degree 2(p-1) by rows.
+constexpr int kTapWords = 16, kFWords = 12;
+__host__ __device__ constexpr int screen_form_words(int p) {
+  return (tri(2 * (p - 1) + 1) + 1) * rows::pitch_of(2 * (p - 1));
 }
-__host__ __device__ constexpr int screen_warp_bytes(int max_p) { return 48 + 2 * screen_buf_bytes(max_p); }
-
-// (s, t) of entry i of a slice (entries ordered by s, then t <= s).
-__device__ __forceinline__ void decode_slice_entry(int i, int &s, int &t) {
-  s = (isqrt(8 * i + 1) - 1) >> 1;
-  while (tri(s + 1) <= i) ++s;
-  while (s > 0 && tri(s) > i) --s;
-  t = i - tri(s);
-}
-
-// out = in * f mod p, in of degree m (packed), out of degree m + 4; the warp's lanes split every slice.
-template <int P>
-__device__ void warp_times_f(const uint8_t *in, int m, uint8_t *out, const uint8_t *f, int lane) {
-  const int M = m + 4;
-  for (int u = 0; u <= M; ++u) {
-    const int n = tri(u + 1);
-    int s, t;
-    decode_slice_entry(lane, s, t);
-    for (int i = lane; i < n; i += 32, t += 32) {
-      while (t > s) t -= ++s;   // entry i = tri(s) + t: advance (s, t) by the 32 entries since the last one
-      int acc = 0;
-#pragma unroll
-      for (int uI = 0; uI <= 4; ++uI) {
-        const int ui = u - uI;
-        if (ui < 0 || ui > m) continue;
-#pragma unroll
-        for (int sI = 0; sI <= uI; ++sI) {
-          const int si = s - sI;
-          if (si < 0 || si > ui) continue;
-#pragma unroll
-          for (int tI = 0; tI <= sI; ++tI) {
-            const int ti = t - tI;
-            if (ti < 0 || ti > si) continue;
-            acc += (int)f[tet(uI) + tri(sI) + tI] * (int)in[tet(ui) + tri(si) + ti];
-          }
-        }
-      }
-      out[tet(u) + tri(s) + t] = (uint8_t)(acc % P);
-    }
-  }
-  __syncwarp();
-}
+__host__ __device__ constexpr int screen_warp_words(int max_p) { return kTapWords + kFWords + 2 * screen_form_words(max_p); }
+// words of the list of output words, shared by the CTA's warps
+__host__ __device__ constexpr int screen_item_words(int max_p) { return (rows::items_of(2 * (max_p - 1)) + 1) / 2; }
 
 // Screens one row with the calling warp; returns -1 (a coefficient >= p), 1 (height 1) or 0 (survivor), same in
-// every lane.
+// every lane.  fresh: the region last held forms of another prime (or nothing).
 template <int P>
-__device__ int screen_row(const uint8_t *__restrict__ f35, uint8_t *wsm, int lane) {
-  constexpr int k = (P - 1) / 2;
-  uint8_t *f = wsm;
-  uint8_t *A = wsm + 48;
-  uint8_t *B = A + screen_buf_bytes(P);
+__device__ int screen_row(const uint8_t *__restrict__ f35, uint32_t *wsm, const uint16_t *items, bool fresh, int lane) {
+  constexpr int k = (P - 1) / 2, m = 2 * (P - 1), pitch = rows::pitch_of(m), form = screen_form_words(P);
+  rows::TapWords &T = *reinterpret_cast<rows::TapWords *>(wsm);
+  uint8_t *f = reinterpret_cast<uint8_t *>(wsm + kTapWords);
+  uint32_t *A = wsm + kTapWords + kFWords + pitch, *B = A + form;   // row 0; the words a row does not use stay zero
+  if (fresh)
+    for (int i = lane; i < 2 * form; i += 32) wsm[kTapWords + kFWords + i] = 0u;
   int bad = 0;
   for (int i = lane; i < 35; i += 32) {
     const int a = f35[i];
@@ -80,51 +46,74 @@ __device__ int screen_row(const uint8_t *__restrict__ f35, uint8_t *wsm, int lan
   }
   if (__any_sync(0xffffffffu, bad)) return -1;
   __syncwarp();
-  // F = f^k: f itself is the degree-4 form, then k - 1 products
-  const uint8_t *F = f;
-  for (int j = 1; j < k; ++j) {
-    uint8_t *dst = (j & 1) ? A : B;
-    warp_times_f<P>(F, 4 * j, dst, f, lane);
-    F = dst;
+  if (lane < 15) T.tw[lane] = rows::tap_word(f, lane);
+  if (lane == 15) T.a44 = f[34];
+  // F = f^k: the rows of f, then k - 1 products
+  uint32_t *F = A, *next = B;
+  for (int i = lane; i < 35; i += 32) {
+    int u, s, t;
+    decode_packed(i, u, s, t, 4);
+    reinterpret_cast<uint8_t *>(F + (tri(u) + s) * pitch + 1)[t] = f[i];
   }
-  // coefficient of (x1 x2 x3 x4)^(p-1) in F * F
-  constexpr int m = 2 * (P - 1);
-  int acc = 0;
-  for (int i = lane; i < tet(m + 1); i += 32) {
-    // (u, s, t) of packed entry i of degree m
-    int u = 0;
-    while (tet(u + 1) <= i) ++u;
-    int s, t;
-    decode_slice_entry(i - tet(u), s, t);
-    const int e1 = m - u, e2 = u - s, e3 = s - t, e4 = t;
-    if (e1 <= P - 1 && e2 <= P - 1 && e3 <= P - 1 && e4 <= P - 1) {
-      const int ub = 3 * (P - 1) - u, sb = 2 * (P - 1) - s, tb = (P - 1) - t;
-      acc += (int)F[i] * (int)F[tet(ub) + tri(sb) + tb];
+  __syncwarp();
+  int n_items = rows::items_of(4);
+#pragma unroll 1
+  for (int j = 1; j < k; ++j) {
+#pragma unroll
+    for (int v = 1; v <= 4; ++v) n_items += rows::words_below(4 * j + v + 1);
+    for (int i = lane; i < n_items; i += 32) {
+      int u, s, w;
+      rows::item_of(items, i, u, s, w);
+      uint32_t g[4];
+      rows::word_sums<pitch>(F, 4 * j, T, u, s, w, g);
+      next[(tri(u) + s) * pitch + 1 + w] = g[0] % P | (g[1] % P) << 8 | (g[2] % P) << 16 | (g[3] % P) << 24;
     }
+    __syncwarp();
+    uint32_t *t = F;
+    F = next;
+    next = t;
+  }
+  // coefficient of (x1 x2 x3 x4)^(p-1) in F * F, one row (u, s) per lane
+  int acc = 0;
+  int u = (isqrt(8 * lane + 1) - 1) >> 1, s = lane - tri(u);
+  for (int row = lane; row < tri(m + 1); row += 32, s += 32) {
+    while (s > u) s -= ++u;
+    if (m - u > P - 1 || u - s > P - 1) continue;
+    const uint8_t *x = reinterpret_cast<const uint8_t *>(F + (tri(u) + s) * pitch + 1);
+    const int ub = 3 * (P - 1) - u, sb = 2 * (P - 1) - s;
+    const uint8_t *y = reinterpret_cast<const uint8_t *>(F + (tri(ub) + sb) * pitch + 1) + (P - 1);
+    const int t_hi = min(s, P - 1);
+    for (int t = max(0, s - (P - 1)); t <= t_hi; ++t) acc += (int)x[t] * (int)y[-t];
   }
   acc = __reduce_add_sync(0xffffffffu, acc);
   return (acc % P) != 0 ? 1 : 0;
 }
 
-__global__ void __launch_bounds__(kScreenThreads) screen_kernel(FusedParams prm, int warp_bytes, int64_t *list,
-                                                                unsigned long long *n_list) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+__global__ void __launch_bounds__(kScreenThreads) screen_kernel(const __grid_constant__ FusedParams prm, int max_p,
+                                                                int64_t *list, unsigned long long *n_list) {
+  extern __shared__ __align__(16) uint32_t smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint8_t *wsm = smem_raw + (size_t)warp * warp_bytes;
+  uint16_t *items = reinterpret_cast<uint16_t *>(smem);
+  uint32_t *wsm = smem + screen_item_words(max_p) + (size_t)warp * screen_warp_words(max_p);
+  rows::build_items(items, 2 * (max_p - 1));
+  __syncthreads();
   const int64_t stride = (int64_t)gridDim.x * kScreenWarps;
+  int last_p = 0;   // prime of the forms in the warp's region
   for (int64_t item = (int64_t)blockIdx.x * kScreenWarps + warp; item < prm.n_items; item += stride) {
     int gi = 0;
     while (gi + 1 < prm.n_groups && item >= prm.g[gi + 1].item_begin) ++gi;
     const FusedGroup &G = prm.g[gi];
     const int64_t row = item - G.item_begin;
     const uint8_t *f = G.coeffs + 35 * row;
+    const bool fresh = G.p != last_p;
+    last_p = G.p;
     int r;
     switch (G.p) {
-      case 3: r = screen_row<3>(f, wsm, lane); break;
-      case 5: r = screen_row<5>(f, wsm, lane); break;
-      case 7: r = screen_row<7>(f, wsm, lane); break;
-      case 11: r = screen_row<11>(f, wsm, lane); break;
-      default: r = screen_row<13>(f, wsm, lane); break;
+      case 3: r = screen_row<3>(f, wsm, items, fresh, lane); break;
+      case 5: r = screen_row<5>(f, wsm, items, fresh, lane); break;
+      case 7: r = screen_row<7>(f, wsm, items, fresh, lane); break;
+      case 11: r = screen_row<11>(f, wsm, items, fresh, lane); break;
+      default: r = screen_row<13>(f, wsm, items, fresh, lane); break;
     }
     if (lane == 0) {
       if (r != 0) G.heights[row] = (int8_t)r;
@@ -136,14 +125,16 @@ __global__ void __launch_bounds__(kScreenThreads) screen_kernel(FusedParams prm,
 
 }  // namespace
 
-size_t screen_smem_bytes(int max_p) { return (size_t)kScreenWarps * screen_warp_bytes(max_p); }
+size_t screen_smem_bytes(int max_p) {
+  return sizeof(uint32_t) * ((size_t)screen_item_words(max_p) + (size_t)kScreenWarps * screen_warp_words(max_p));
+}
 
 cudaError_t screen_launch(const FusedParams &prm, int max_p, int64_t *list, unsigned long long *n_list,
                           int grid_ctas, cudaStream_t st) {
   const size_t smem = screen_smem_bytes(max_p);
   cudaError_t e = cudaFuncSetAttribute(screen_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  screen_kernel<<<grid_ctas, kScreenThreads, smem, st>>>(prm, screen_warp_bytes(max_p), list, n_list);
+  screen_kernel<<<grid_ctas, kScreenThreads, smem, st>>>(prm, max_p, list, n_list);
   return cudaGetLastError();
 }
 
