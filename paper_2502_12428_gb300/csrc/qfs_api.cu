@@ -41,6 +41,8 @@ struct DeviceState {
   size_t mm_bytes = 0;
   void *pp = nullptr;          // polynomial powering: transform, twiddles, residues, input
   size_t pp_bytes = 0;
+  void *classes = nullptr;     // theta by rows (p <= 5): the classes of every CTA
+  size_t classes_bytes = 0;
   void *list = nullptr;        // survivors of the height-1 screen (int64 launch items)
   size_t list_bytes = 0;
 };
@@ -128,6 +130,23 @@ int ensure_list(DeviceState &S, size_t bytes) {
     return QFS_ERR_NO_MEMORY;
   }
   S.list_bytes = bytes;
+  return QFS_OK;
+}
+
+int ensure_classes(DeviceState &S, size_t bytes) {
+  if (S.classes_bytes >= bytes) return QFS_OK;
+  if (S.classes) {
+    cudaError_t e = cudaFree(S.classes);
+    S.classes = nullptr;
+    S.classes_bytes = 0;
+    if (e != cudaSuccess) return cuda_fail(e);
+  }
+  if (cudaMalloc(&S.classes, bytes) != cudaSuccess) {
+    S.classes = nullptr;
+    (void)cudaGetLastError();
+    return QFS_ERR_NO_MEMORY;
+  }
+  S.classes_bytes = bytes;
   return QFS_OK;
 }
 
@@ -259,6 +278,7 @@ int mixed_crew(const FusedParams &prm, int slots) {
 struct Plan {
   int grid = 0;        // CTAs of a launch without crews
   int crews[4] = {};   // crews of 2^i CTAs the device holds at once (0: not used)
+  int64_t ctas = 0;    // CTAs that need buffers
   size_t smem = 0;
   size_t ws_words = 0;
 };
@@ -301,6 +321,7 @@ int make_plan(DeviceState &S, int form, int max_p, int64_t n_items, const qfs_op
   grid = std::min<int64_t>(grid, n_items);
   if (grid < 1) return QFS_ERR_NO_MEMORY;
   plan.grid = (int)grid;
+  plan.ctas = ctas;
   return ensure_workspace(S, workspace_words(ctas, plan.ws_words) * sizeof(uint32_t));
 }
 
@@ -417,6 +438,19 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
   prm.stats = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(S->ctrl) + 16);
   prm.ws = reinterpret_cast<uint32_t *>(S->ws);
   prm.ws_words = plan.ws_words;
+  // theta by rows for the groups with p <= 5, unless the budget does not cover the classes as well
+  if (power == QFS_POWER_CHAIN) {
+    size_t words = 0;
+    for (int i = 0; i < prm.n_groups; ++i) words = std::max(words, row_class_words(prm.g[i].p));
+    const size_t bytes = words * sizeof(uint32_t) * (size_t)plan.ctas;
+    const size_t budget = opts && opts->workspace_budget ? opts->workspace_budget : default_budget(*S);
+    if (words && bytes + workspace_words(plan.ctas, plan.ws_words) * sizeof(uint32_t) <= budget) {
+      rc = ensure_classes(*S, bytes);
+      if (rc) return rc;
+      prm.classes = static_cast<uint32_t *>(S->classes);
+      prm.class_words = words;
+    }
+  }
   // height-1 screen first: the persistent launch then runs only the quartics that pass it
   rc = ensure_list(*S, (size_t)n_items * sizeof(int64_t));
   if (rc) return rc;
@@ -480,6 +514,10 @@ int qfs_plan_prepare(int p, int64_t n_hint) {
                         4 * (size_t)ring_words_for(p, tile_for(p), uses_ring_chain(QFS_FORM_DP4A, p), QFS_POWER_CHAIN);
     rc = make_plan(*S, QFS_FORM_DP4A, p, n, nullptr, plan, smem, &prm);
     if (rc) return rc;
+    if (row_class_words(p)) {
+      rc = ensure_classes(*S, row_class_words(p) * sizeof(uint32_t) * (size_t)plan.ctas);
+      if (rc) return rc;
+    }
   }
   if (n_hint > 0) {
     rc = ensure_list(*S, (size_t)n_hint * sizeof(int64_t));
@@ -505,6 +543,7 @@ int qfs_shutdown(void) {
     if (S.mm && cudaFree(S.mm) != cudaSuccess) rc = QFS_ERR_CUDA;
     if (S.pp && cudaFree(S.pp) != cudaSuccess) rc = QFS_ERR_CUDA;
     if (S.list && cudaFree(S.list) != cudaSuccess) rc = QFS_ERR_CUDA;
+    if (S.classes && cudaFree(S.classes) != cudaSuccess) rc = QFS_ERR_CUDA;
     S = DeviceState();
   }
   cudaSetDevice(cur);

@@ -22,6 +22,7 @@
 #include "qfs_common.cuh"
 #include "qfs_sweep.cuh"
 #include "qfs_block.cuh"
+#include "qfs_theta_rows.cuh"
 
 namespace qfs {
 
@@ -601,6 +602,8 @@ inline size_t theta_class_words(int p) {
   return b / 4;
 }
 
+__host__ __device__ constexpr int max_of(int a, int b) { return a > b ? a : b; }
+
 // Ring words of theta for one power mode (-1: every mode).  At p = 7 the chain mode streams (theta_stream) and
 // the identity mode runs by classes; the reduced mode keeps its arrays in the power modes' part of the ring.
 template <int P>
@@ -611,7 +614,8 @@ __host__ __device__ constexpr int theta_ring_words(int power = -1) {
       constexpr int stream = theta_stream_ring_words<P>();
       return power == 0 ? stream : power == 1 ? poly : power == 2 ? 0 : (poly > stream ? poly : stream);
     } else {
-      return power == 2 ? 0 : poly;
+      constexpr int by_rows = row_class_smem_words(P);   // the chain mode, where the launch has room for the classes
+      return power == 2 ? 0 : max_of(by_rows, poly);
     }
   } else {
     return (theta_r_words<P>() + 4 * (P - 1) + 2 + 3) & ~3;   // reversed g columns and their slice table
@@ -1142,6 +1146,20 @@ __device__ __noinline__ void chain_step_call(const uint32_t *in, uint32_t *out, 
   chain_step<P, FORM, false, DEBUG>(in, out, m_in, sm, ring, gs, status, dbg);
 }
 
+// Tap words and the mask of nonzero pairs from sm.taps, by the first warp; the caller synchronises before and after.
+__device__ __forceinline__ void build_tap_words(Smem &sm) {
+  if (threadIdx.x < 32) {
+    const int pi = (int)threadIdx.x;
+    uint32_t w = 0;
+    if (pi < 15) {
+      w = rows::tap_word(sm.taps, pi);
+      sm.tapword[pi] = w;
+    }
+    const uint32_t mask = __ballot_sync(0xffffffffu, w != 0 || (pi == 14 && sm.taps[34] != 0));
+    if (pi == 0) sm.pair_mask = mask;
+  }
+}
+
 // A1: read the 35 coefficients into the tap tables; returns false (after a barrier) if one is >= p.
 template <int P>
 __device__ __forceinline__ bool setup_quartic(const uint8_t *__restrict__ f35, Smem &sm) {
@@ -1156,26 +1174,12 @@ __device__ __forceinline__ bool setup_quartic(const uint8_t *__restrict__ f35, S
   block::build_strip_tab(P, sm);
   if (tid < 2) sm.unit_next[tid] = 0;
   if (__syncthreads_or(bad)) return false;
-  if (tid == 0) {
-    uint32_t mask = 0;
-    for (int uI = 0; uI <= 4; ++uI)
-      for (int sI = 0; sI <= uI; ++sI) {
-        uint32_t tw = 0;
-        bool nz = false;
-        for (int tI = 0; tI <= sI; ++tI) {
-          const int a = sm.taps[tet(uI) + tri(sI) + tI];
-          nz |= a != 0;
-          if (tI <= 3) tw |= (uint32_t)a << (8 * (3 - tI));
-        }
-        sm.tapword[tri(uI) + sI] = tw;
-        if (nz) mask |= 1u << (tri(uI) + sI);
-      }
-    sm.pair_mask = mask;
-    for (int c = 0; c < P; ++c) {
-      int v = 1;
-      for (int e = 0; e < P; ++e) v = (v * c) % Pr::p2;
-      sm.powp[c] = v;
-    }
+  build_tap_words(sm);
+  if (tid >= 32 && tid < 32 + P) {
+    const int c = tid - 32;
+    int v = 1;
+    for (int e = 0; e < P; ++e) v = (v * c) % Pr::p2;
+    sm.powp[c] = v;
   }
   return true;
 }
@@ -1377,22 +1381,7 @@ __device__ __noinline__ uint32_t *power_identity(Smem &sm, const uint8_t *gs, ui
   // A~ (coefficients a~_I^p mod p^2) into cur, then A~^(p-1) mod p^2 by p-2 chain products (ping-pong inside cur)
   if (tid < 35) sm.taps[tid] = sm.powp[sm.taps[tid]];
   __syncthreads();
-  if (tid == 0) {
-    uint32_t mask = 0;
-    for (int uI = 0; uI <= 4; ++uI)
-      for (int sI = 0; sI <= uI; ++sI) {
-        uint32_t tw = 0;
-        bool nz = false;
-        for (int tI = 0; tI <= sI; ++tI) {
-          const int a = sm.taps[tet(uI) + tri(sI) + tI];
-          nz |= a != 0;
-          if (tI <= 3) tw |= (uint32_t)a << (8 * (3 - tI));
-        }
-        sm.tapword[tri(uI) + sI] = tw;
-        if (nz) mask |= 1u << (tri(uI) + sI);
-      }
-    sm.pair_mask = mask;
-  }
+  build_tap_words(sm);
   // pa = cur, pb after pa's largest form and a guard of zero words (chain products read from both)
   uint32_t *pa = cur, *pb = cur + sm.SW[d + 1] + kGuardWords;
   if (tid < kGuardWords) pb[tid - kGuardWords] = 0u;
@@ -1596,11 +1585,13 @@ __device__ __noinline__ int reduced_height(Smem &sm, uint8_t *gs, uint8_t *gn, u
 }
 
 // Runs A1-A7 for one quartic with the CTA's two workspace buffers; returns the height code.  crewA: the first of the
-// crew's buffers if the CTA belongs to one (chain power mode, dp4a form), else null.
+// crew's buffers if the CTA belongs to one (chain power mode, dp4a form), else null.  classes: row_class_words(p) words of
+// this CTA for theta by rows at p <= 5 (chain power mode), or null.
 template <int P, int FORM, bool DEBUG>
 __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem &sm, uint8_t *gs, uint8_t *gn,
                                uint32_t *ring, uint32_t *bufA, uint32_t *bufB, uint32_t *status, DebugPtrs dbg,
-                               int &theta_steps, int power_mode = 0, uint32_t *crewA = nullptr) {
+                               int &theta_steps, int power_mode = 0, uint32_t *crewA = nullptr,
+                               uint32_t *classes = nullptr) {
   using Pr = Prime<P>;
   const int tid = threadIdx.x;
   theta_steps = 0;
@@ -1647,9 +1638,12 @@ __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem 
   uint32_t *dg = delta == bufA ? bufB : bufA;
   unsigned char *ringb = reinterpret_cast<unsigned char *>(ring);
   const bool by_classes = theta_by_classes<P>() && (!theta_streams<P>() || in_classes);
+  const bool by_rows = P <= 5 && classes != nullptr && !in_classes;
   if constexpr (theta_by_classes<P>()) {
     if (in_classes) {
       dg = delta;
+    } else if (by_rows) {
+      if constexpr (P <= 5) delta_to_rows<P>(delta, classes, sm, ring);
     } else if (by_classes) {
       // (theta by classes is not split: each CTA of a crew makes its own copy, in its own order of classes)
       if (sm.rank != 0) dg = own;
@@ -1664,7 +1658,9 @@ __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem 
   for (int h = 2; h <= max_h; ++h) {
     bool nonzero;
     if constexpr (theta_by_classes<P>()) {
-      if (by_classes) nonzero = theta_poly<P>(dg, g, g2, ringb);
+      if constexpr (P <= 5) {
+        nonzero = by_rows ? theta_rows<P>(classes, g, g2, ring) : theta_poly<P>(dg, g, g2, ringb);
+      } else if (by_classes) nonzero = theta_poly<P>(dg, g, g2, ringb);
       else nonzero = theta_stream<P>(delta, sm, g, g2, ring);
     } else {
       nonzero = theta_gather<P>(dg, sm, g, g2, ring);
@@ -1704,6 +1700,8 @@ struct FusedParams {
   unsigned long long *stats;          // [0] quartics past the height-1 test, [1] theta steps run
   uint32_t *ws;                       // workspace: a guard, then 2 buffers of ws_words (the stride) per CTA
   size_t ws_words;
+  uint32_t *classes;                  // per CTA class_words words for theta by rows (p <= 5, chain mode), or null
+  size_t class_words;
   int crew;                           // CTAs per cluster of the launch (1: no clusters)
   int64_t run_min, run_max;           // the launch does nothing unless the items to run are run_min .. run_max
   int power_mode;                     // 0: chain (Algorithm 1 literally), 1: identity shortcut, 2: reduced theta
@@ -1731,6 +1729,7 @@ __device__ __forceinline__ void fused_body(const FusedParams &prm) {
   cta_buffers(prm.ws, prm.ws_words, bufA, bufB);
   DebugPtrs dbg{nullptr, nullptr, nullptr, nullptr};
   const int crew = FORM == 1 ? prm.crew : 1, rank = crew > 1 ? crew_rank() : 0;
+  uint32_t *classes = prm.classes ? prm.classes + (size_t)blockIdx.x * prm.class_words : nullptr;
   uint32_t *crewA = crew > 1 ? bufA - (size_t)rank * 2 * prm.ws_words : nullptr;
   for (;;) {
     crew_sync(crew);
@@ -1759,16 +1758,16 @@ __device__ __forceinline__ void fused_body(const FusedParams &prm) {
     const uint8_t *f = G.coeffs + 35 * row;
     int h, steps;
     switch (G.p) {
-      case 3: h = process_quartic<3, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA); break;
-      case 5: h = process_quartic<5, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA); break;
+      case 3: h = process_quartic<3, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA, classes); break;
+      case 5: h = process_quartic<5, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA, classes); break;
       default:
         if constexpr (SMALL) {
           h = -1;   // not reached: the host launches the small-prime kernel only when every group has p <= 5
         } else {
           switch (G.p) {
-            case 7: h = process_quartic<7, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA); break;
-            case 11: h = process_quartic<11, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA); break;
-            default: h = process_quartic<13, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA); break;
+            case 7: h = process_quartic<7, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA, classes); break;
+            case 11: h = process_quartic<11, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA, classes); break;
+            default: h = process_quartic<13, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA, classes); break;
           }
         }
         break;

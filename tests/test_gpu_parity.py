@@ -248,6 +248,21 @@ def test_theta_matrix_by_crews_repeats(qfs):
     assert qfs.read_status() == 0
 
 
+# ------------------------------------------------------------------------------------- theta by rows
+@pytest.mark.parametrize("p,n", [(3, 4000), (5, 6000)])
+@pytest.mark.parametrize("form", CORE_FORMS)
+def test_theta_by_rows_many_steps(qfs, p, n, form):
+    # sparse quartics run up to nine theta steps; a workspace budget without room for the classes takes theta by cubes,
+    # with the same heights
+    f = inputs.sparse(p, n, 9900 + p)
+    want = oracle.heights(p, f)
+    assert len(set(want.tolist())) >= 5 and (want > 3).any()
+    t = dev_tensor(f)
+    assert np.array_equal(qfs.heights(p, t, form=form).cpu().numpy(), want)
+    assert np.array_equal(qfs.heights(p, t, form=form, workspace_budget=1 << 20).cpu().numpy(), want)
+    assert qfs.read_status() == 0
+
+
 # ------------------------------------------------------------------------------------- edge cases and errors
 def test_edge_cases(qfs):
     p = 5
