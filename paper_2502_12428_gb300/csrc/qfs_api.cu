@@ -250,28 +250,28 @@ bool form_supported(int form) { return form == QFS_FORM_INT32 || form == QFS_FOR
 
 // Crews (clusters of CTAs per quartic, see qfs_common.cuh) of a dp4a chain launch at p >= 7.  One CTA per quartic is the
 // best use of the device while there are many; with few quartics past height 1, or with a few heavy ones (p = 11 beside
-// p = 5), CTAs run out of work while others are in the middle of a quartic.  A crew of 8 takes 0.56 ms for a quartic at
-// p = 7 that one CTA takes 2.2 ms for alone, but 300 quartics take 6.2 ms by crews of 8 and 4.4 ms by single CTAs, so the largest
-// crew that leaves every quartic one at once is taken (1,001 random quartics at p = 7: 6.1 -> 3.1 to 3.7 ms with the block
-// products, 5.4 ms without crews; 48 theta matrices: 3.1 -> 2.2 ms; p = 5, 7 and 11 together, 47 heavy quartics: 204 -> 83 ms).
-//   One prime: the number of survivors decides on the device.  A launch is made for each crew size that can come up,
-// and all but one find that it is not their turn.
-//   Several primes: estimated here from the share 1/p of quartics past height 1 and the outputs of their chains: the heaviest quartic
-// should take at most half of what the launch takes if its work is spread evenly.
+// p = 5), CTAs run out of work while others are in the middle of a quartic.  1,001 random quartics at p = 7 take 5.4 ms
+// without crews and 3.2 ms with them, 48 theta matrices 3.1 and 2.2 ms, p = 5, 7 and 11 together (47 quartics
+// of p = 11 past height 1) 204 and 83 ms.
+//   One prime: the number of survivors decides on the device (crew_for).  A launch is made for each crew size that can
+// come up, and all but one find that it is not their turn.
+//   Several primes: one size, estimated here from the share 1/p of quartics past height 1 and the outputs of their
+// chains: the heaviest quartic should take at most half of what the launch takes if its work is spread evenly.
 bool same_prime(const FusedParams &prm) {
   for (int i = 1; i < prm.n_groups; ++i)
     if (prm.g[i].p != prm.g[0].p) return false;
   return true;
 }
 int mixed_crew(const FusedParams &prm, int slots) {
-  const double outputs[kMaxP + 1] = {0, 0, 0, 2e4, 0, 4.3e5, 0, 8.3e6, 0, 0, 0, 4e8, 0, 1.6e9};
-  double work = 0, heaviest = 0;
+  const int64_t outputs[kMaxP + 1] = {0, 0, 0, 20000, 0, 430000, 0, 8300000, 0, 0, 0, 400000000, 0, 1600000000};
+  int64_t work = 0, heaviest = 0;
   for (int i = 0; i < prm.n_groups; ++i) {
     const int p = prm.g[i].p;
-    work += outputs[p] * std::max(1.0, (double)prm.g[i].n / p);
+    const int64_t rows = std::min<int64_t>(std::max<int64_t>(1, prm.g[i].n / p), 1 << 20);
+    work += outputs[p] * rows;
     heaviest = std::max(heaviest, outputs[p]);
   }
-  const double need = 2 * slots * heaviest / work;
+  const int64_t need = 2 * slots * heaviest / work;
   return need >= 8 ? 8 : need >= 4 ? 4 : need >= 2 ? 2 : 1;
 }
 
@@ -307,7 +307,7 @@ int make_plan(DeviceState &S, int form, int max_p, int64_t n_items, const qfs_op
     const bool one_prime = same_prime(*prm);
     const int want = one_prime ? 0 : mixed_crew(*prm, (int)grid);
     // a batch of one prime with many rows will not leave few survivors
-    const bool few = one_prime && n_items / max_p <= 2 * grid;
+    const bool few = one_prime && n_items / max_p <= 3 * grid;
     for (int i = 1; i < 4; ++i) {
       const int crew = 1 << i;
       if (one_prime ? !few : crew != want) continue;
@@ -462,19 +462,13 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
   prm.list = static_cast<const int64_t *>(S->list);
   prm.n_list = n_list;
   if (reduced_p) return (e = reduced_launch(reduced_p, prm, S->sms, stream)) == cudaSuccess ? QFS_OK : cuda_fail(e);
-  int crews_at_once = 0;   // of the larger crews: up to so many survivors are theirs
-  for (int i = 3; i >= 0; --i) {
-    const int at_once = i > 0 ? plan.crews[i] : plan.grid;
-    if (at_once == 0) continue;
-    const bool last = i == 0 || !one_prime;   // several primes: one crew size, whatever the number of survivors
+  for (int i = 0; i < 4; ++i) prm.crews[i] = plan.crews[i];
+  if (one_prime || std::max({plan.crews[1], plan.crews[2], plan.crews[3]}) == 0) prm.crews[0] = plan.grid;
+  for (int i = 0; i < 4; ++i) {
+    if (prm.crews[i] == 0) continue;
     prm.crew = 1 << i;
-    prm.run_min = crews_at_once + 1;
-    prm.run_max = last ? INT64_MAX : at_once;
-    if (prm.run_min > n_items || prm.run_max < prm.run_min) continue;
-    e = form_fused(form, prm, i > 0 ? at_once << i : at_once, plan.smem, stream, form == QFS_FORM_INT8TC && max_p <= 5);
+    e = form_fused(form, prm, prm.crews[i] << i, plan.smem, stream, form == QFS_FORM_INT8TC && max_p <= 5);
     if (e != cudaSuccess) return cuda_fail(e);
-    if (last) break;
-    crews_at_once = at_once;
   }
   return QFS_OK;
 }

@@ -1703,11 +1703,24 @@ struct FusedParams {
   uint32_t *classes;                  // per CTA class_words words for theta by rows (p <= 5, chain mode), or null
   size_t class_words;
   int crew;                           // CTAs per cluster of the launch (1: no clusters)
-  int64_t run_min, run_max;           // the launch does nothing unless the items to run are run_min .. run_max
+  int crews[4];                       // crews of 2^i CTAs that run at once (0: no such launch is made); see crew_for
   int power_mode;                     // 0: chain (Algorithm 1 literally), 1: identity shortcut, 2: reduced theta
   const int64_t *list;                // if set: the items to run (the survivors of the height-1 screen) ...
   const unsigned long long *n_list;   // ... and their count; if null, every item 0 .. n_items-1 runs
 };
+
+// The crew size for n_run quartics of one prime, among those that launches are made for.  Crews of 8 while each quartic
+// gets one at once, smaller ones for up to three rounds, as measured at p = 7 with random quartics of height >= 2 (ms per
+// call by crews of 1, 2, 4 and 8; 304, 152, 76 and 38 run at once):
+//     36: 3.7, 2.1, 1.2, 1.0     100: 3.7, 2.8, 2.4, 2.7     160: 5.1, 4.1, 3.6, 4.1     250: 5.3, 5.2, 4.9, 6.0
+//     310: 7.0, 6.3, 6.1, 7.3    400: 8.0, 7.6, 7.6, 9.4     600: 10.4, 10.6, 11.4, 13.8
+__host__ __device__ inline int crew_for(int64_t n_run, const int (&crews)[4]) {
+  if (n_run <= crews[3]) return 8;
+  if (n_run <= 3 * (int64_t)crews[2]) return 4;
+  if (n_run <= 3 * (int64_t)crews[1]) return 2;
+  if (crews[0] > 0) return 1;
+  return crews[1] > 0 ? 2 : crews[2] > 0 ? 4 : 8;   // several primes: the only one there is
+}
 
 // SMALL: an int8 tensor form launch whose primes are all <= 5; the kernel then needs no code for larger primes and
 // can keep three CTAs per SM.
@@ -1715,7 +1728,7 @@ template <int FORM, bool SMALL>
 __device__ __forceinline__ void fused_body(const FusedParams &prm) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int64_t n_run = prm.list ? (int64_t)*prm.n_list : prm.n_items;
-  if (FORM == 1 && (n_run < prm.run_min || n_run > prm.run_max)) return;
+  if (FORM == 1 && crew_for(n_run, prm.crews) != prm.crew) return;   // another launch's turn
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
   uint8_t *gs = smem_raw + sizeof(Smem);
   // the second iterate buffer follows the largest ld in this launch

@@ -148,7 +148,7 @@ extern "C" int qfs_heights_noalloc(int p, int64_t n, const uint8_t *coeffs, int 
   prm.ws = reinterpret_cast<uint32_t *>(base + kControlBytes);
   prm.ws_words = ws_words;
   prm.crew = 1;
-  prm.run_max = n;
+  prm.crews[0] = 1;
   prm.power_mode = QFS_POWER_CHAIN;
   // The array keeps whatever the previous call left.  Only the work-queue counter must start at zero; the check
   // word and the work counters accumulate until qfs_read_status / qfs_read_stats take them.  The chain buffers
