@@ -41,8 +41,7 @@ struct DeviceState {
   size_t mm_bytes = 0;
   void *pp = nullptr;          // polynomial powering: transform, twiddles, residues, input
   size_t pp_bytes = 0;
-  void *classes = nullptr;     // theta by rows (p <= 5): the classes of every CTA
-  size_t classes_bytes = 0;
+  void *classes[3] = {};       // theta by rows at p = 3, 5, 7: the classes of class_ctas CTAs
   void *list = nullptr;        // survivors of the height-1 screen (int64 launch items)
   size_t list_bytes = 0;
 };
@@ -133,21 +132,22 @@ int ensure_list(DeviceState &S, size_t bytes) {
   return QFS_OK;
 }
 
-int ensure_classes(DeviceState &S, size_t bytes) {
-  if (S.classes_bytes >= bytes) return QFS_OK;
-  if (S.classes) {
-    cudaError_t e = cudaFree(S.classes);
-    S.classes = nullptr;
-    S.classes_bytes = 0;
-    if (e != cudaSuccess) return cuda_fail(e);
+// The classes' buffer of prime p: one size per prime, kept until qfs_shutdown, so that launches in flight and captured
+// graphs never lose it; null if the memory is not there.  The first call may come during a stream capture whose
+// workspace was prepared, so the allocation is made in relaxed mode, which a capture allows.
+int64_t class_ctas(const DeviceState &S, int p) { return (int64_t)S.sms * (p == 7 ? 2 : 4); }
+uint32_t *ensure_classes(DeviceState &S, int p) {
+  void *&c = S.classes[(p - 3) / 2];
+  if (!c) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
+    if (cudaMalloc(&c, row_class_words(p) * sizeof(uint32_t) * (size_t)class_ctas(S, p)) != cudaSuccess) {
+      c = nullptr;
+      (void)cudaGetLastError();
+    }
+    (void)cudaThreadExchangeStreamCaptureMode(&mode);
   }
-  if (cudaMalloc(&S.classes, bytes) != cudaSuccess) {
-    S.classes = nullptr;
-    (void)cudaGetLastError();
-    return QFS_ERR_NO_MEMORY;
-  }
-  S.classes_bytes = bytes;
-  return QFS_OK;
+  return static_cast<uint32_t *>(c);
 }
 
 // Default workspace budget: a quarter of device memory.
@@ -438,17 +438,16 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
   prm.stats = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(S->ctrl) + 16);
   prm.ws = reinterpret_cast<uint32_t *>(S->ws);
   prm.ws_words = plan.ws_words;
-  // theta by rows for the groups with p <= 5, unless the budget does not cover the classes as well
-  if (power == QFS_POWER_CHAIN) {
-    size_t words = 0;
-    for (int i = 0; i < prm.n_groups; ++i) words = std::max(words, row_class_words(prm.g[i].p));
-    const size_t bytes = words * sizeof(uint32_t) * (size_t)plan.ctas;
+  // theta by rows, unless the budget does not cover the classes as well; without them it runs by cubes
+  int class_p = 0;
+  for (int i = 0; i < prm.n_groups; ++i)
+    if (theta_by_rows(prm.g[i].p, power)) class_p = std::max(class_p, prm.g[i].p);
+  if (class_p && plan.ctas <= class_ctas(*S, class_p)) {
+    const size_t bytes = row_class_words(class_p) * sizeof(uint32_t) * (size_t)plan.ctas;
     const size_t budget = opts && opts->workspace_budget ? opts->workspace_budget : default_budget(*S);
-    if (words && bytes + workspace_words(plan.ctas, plan.ws_words) * sizeof(uint32_t) <= budget) {
-      rc = ensure_classes(*S, bytes);
-      if (rc) return rc;
-      prm.classes = static_cast<uint32_t *>(S->classes);
-      prm.class_words = words;
+    if (bytes + workspace_words(plan.ctas, plan.ws_words) * sizeof(uint32_t) <= budget) {
+      prm.classes = ensure_classes(*S, class_p);
+      prm.class_words = row_class_words(class_p);
     }
   }
   // height-1 screen first: the persistent launch then runs only the quartics that pass it
@@ -508,10 +507,6 @@ int qfs_plan_prepare(int p, int64_t n_hint) {
                         4 * (size_t)ring_words_for(p, tile_for(p), uses_ring_chain(QFS_FORM_DP4A, p), QFS_POWER_CHAIN);
     rc = make_plan(*S, QFS_FORM_DP4A, p, n, nullptr, plan, smem, &prm);
     if (rc) return rc;
-    if (row_class_words(p)) {
-      rc = ensure_classes(*S, row_class_words(p) * sizeof(uint32_t) * (size_t)plan.ctas);
-      if (rc) return rc;
-    }
   }
   if (n_hint > 0) {
     rc = ensure_list(*S, (size_t)n_hint * sizeof(int64_t));
@@ -537,7 +532,8 @@ int qfs_shutdown(void) {
     if (S.mm && cudaFree(S.mm) != cudaSuccess) rc = QFS_ERR_CUDA;
     if (S.pp && cudaFree(S.pp) != cudaSuccess) rc = QFS_ERR_CUDA;
     if (S.list && cudaFree(S.list) != cudaSuccess) rc = QFS_ERR_CUDA;
-    if (S.classes && cudaFree(S.classes) != cudaSuccess) rc = QFS_ERR_CUDA;
+    for (void *c : S.classes)
+      if (c && cudaFree(c) != cudaSuccess) rc = QFS_ERR_CUDA;
     S = DeviceState();
   }
   cudaSetDevice(cur);

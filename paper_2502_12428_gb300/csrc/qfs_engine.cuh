@@ -612,9 +612,10 @@ __host__ __device__ constexpr int theta_ring_words(int power = -1) {
     constexpr int poly = (Poly<P>::bytes + 3) / 4;
     if constexpr (theta_streams<P>()) {
       constexpr int stream = theta_stream_ring_words<P>();
-      return power == 0 ? stream : power == 1 ? poly : power == 2 ? 0 : (poly > stream ? poly : stream);
+      constexpr int classes = max_of(poly, row_class_smem_words(P));
+      return power == 0 ? stream : power == 1 ? classes : power == 2 ? 0 : max_of(classes, stream);
     } else {
-      constexpr int by_rows = row_class_smem_words(P);   // the chain mode, where the launch has room for the classes
+      constexpr int by_rows = row_class_smem_words(P);   // where the launch has room for the classes
       return power == 2 ? 0 : max_of(by_rows, poly);
     }
   } else {
@@ -1338,7 +1339,8 @@ __device__ __noinline__ void identity_classes(const uint8_t *__restrict__ fpm2_g
 // f^(p-2)(x^p) Delta_1(f) -- against 2.9e8 for the chain.
 template <int P, int FORM, bool DEBUG>
 __device__ __noinline__ uint32_t *power_identity(Smem &sm, const uint8_t *gs, uint32_t *ring, uint32_t *cur,
-                                                    uint32_t *other, uint32_t *status, DebugPtrs dbg) {
+                                                    uint32_t *other, uint32_t *status, DebugPtrs dbg,
+                                                    uint32_t *classes) {
   using Pr = Prime<P>;
   constexpr int d = Pr::d, D = Pr::D, dm = 4 * (P - 2), d1 = 4 * P;
   constexpr int l_fpm2 = tet(dm + 1), l_d1f = tet(d1 + 1), l_E = Pr::ld;
@@ -1414,8 +1416,12 @@ __device__ __noinline__ uint32_t *power_identity(Smem &sm, const uint8_t *gs, ui
   }
   __syncthreads();
   if constexpr (theta_by_classes<P>()) {
-    // Delta straight into theta's class order, in `cur` (the products above are done with it)
+    // Delta straight into theta's classes, by rows or in class order in `cur` (the products above are done with it)
     if (bad) atomicOr(status, kStatusInexactDivision);
+    if (classes) {
+      identity_rows<P>(fpm2_g, d1f_g, E_g, classes, ring);
+      return cur;
+    }
     unsigned char *ringb = reinterpret_cast<unsigned char *>(ring);
     poly_tables<P>(ringb);
     identity_classes<P, DEBUG>(fpm2_g, d1f_g, E_g, cur, sm, ringb, dbg);
@@ -1586,7 +1592,7 @@ __device__ __noinline__ int reduced_height(Smem &sm, uint8_t *gs, uint8_t *gn, u
 
 // Runs A1-A7 for one quartic with the CTA's two workspace buffers; returns the height code.  crewA: the first of the
 // crew's buffers if the CTA belongs to one (chain power mode, dp4a form), else null.  classes: row_class_words(p) words of
-// this CTA for theta by rows at p <= 5 (chain power mode), or null.
+// this CTA where theta_by_rows, or null.
 template <int P, int FORM, bool DEBUG>
 __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem &sm, uint8_t *gs, uint8_t *gn,
                                uint32_t *ring, uint32_t *bufA, uint32_t *bufB, uint32_t *status, DebugPtrs dbg,
@@ -1624,21 +1630,21 @@ __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem 
   uint32_t *delta;
   // the identity mode at p <= 7 leaves Delta already in theta's class order (and the debug copy written)
   const bool in_classes = power_mode == 1 && theta_by_classes<P>();
+  const bool by_rows = classes != nullptr && theta_by_rows(P, power_mode);
   if (power_mode == 1) {
-    delta = power_identity<P, FORM, DEBUG>(sm, gs, ring, cur, other, status, dbg);
+    delta = power_identity<P, FORM, DEBUG>(sm, gs, ring, cur, other, status, dbg, by_rows ? classes : nullptr);
   } else {
     delta = (nsteps % 2) ? other : cur;
     power_to_G<P, FORM, true, DEBUG>(sm, gs, ring, cur, other, nullptr, status, dbg);
   }
   if (DEBUG && !in_classes)
     for (int k = tid; k < sm.SW[Pr::D + 1]; k += blockDim.x) dbg.delta[k] = delta[k];
-  // A6 + A7.  Theta: by residue classes at p <= 5 and for the identity mode at p = 7 (Delta in class order, copied
-  // into the buffer that does not hold Delta unless the identity mode wrote it so), streamed from the padded Delta
-  // at p = 7 otherwise, and gathered from a guarded copy at p >= 11
+  // A6 + A7.  Theta: by residue classes at p <= 5 and for the identity mode at p = 7 (by rows in `classes`; without
+  // them in class order, copied into the buffer that does not hold Delta unless the identity mode wrote it so), streamed
+  // from the padded Delta at p = 7 otherwise, and gathered from a guarded copy at p >= 11
   uint32_t *dg = delta == bufA ? bufB : bufA;
   unsigned char *ringb = reinterpret_cast<unsigned char *>(ring);
   const bool by_classes = theta_by_classes<P>() && (!theta_streams<P>() || in_classes);
-  const bool by_rows = P <= 5 && classes != nullptr && !in_classes;
   if constexpr (theta_by_classes<P>()) {
     if (in_classes) {
       dg = delta;
@@ -1658,9 +1664,8 @@ __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem 
   for (int h = 2; h <= max_h; ++h) {
     bool nonzero;
     if constexpr (theta_by_classes<P>()) {
-      if constexpr (P <= 5) {
-        nonzero = by_rows ? theta_rows<P>(classes, g, g2, ring) : theta_poly<P>(dg, g, g2, ringb);
-      } else if (by_classes) nonzero = theta_poly<P>(dg, g, g2, ringb);
+      if (by_rows) nonzero = theta_rows<P>(classes, g, g2, ring);
+      else if (by_classes) nonzero = theta_poly<P>(dg, g, g2, ringb);
       else nonzero = theta_stream<P>(delta, sm, g, g2, ring);
     } else {
       nonzero = theta_gather<P>(dg, sm, g, g2, ring);
@@ -1700,7 +1705,7 @@ struct FusedParams {
   unsigned long long *stats;          // [0] quartics past the height-1 test, [1] theta steps run
   uint32_t *ws;                       // workspace: a guard, then 2 buffers of ws_words (the stride) per CTA
   size_t ws_words;
-  uint32_t *classes;                  // per CTA class_words words for theta by rows (p <= 5, chain mode), or null
+  uint32_t *classes;                  // per CTA class_words words for theta by rows, or null
   size_t class_words;
   int crew;                           // CTAs per cluster of the launch (1: no clusters)
   int crews[4];                       // crews of 2^i CTAs that run at once (0: no such launch is made); see crew_for

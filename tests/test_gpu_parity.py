@@ -263,6 +263,35 @@ def test_theta_by_rows_many_steps(qfs, p, n, form):
     assert qfs.read_status() == 0
 
 
+@pytest.mark.parametrize("p,n", [(3, 3000), (5, 4000), (7, 600)])
+@pytest.mark.parametrize("form", CORE_FORMS)
+def test_identity_theta_by_rows(qfs, p, n, form):
+    # the identity mode forms its classes by rows, with and without room for them; sparse quartics need many steps
+    f = np.concatenate([inputs.dense(p, n // 2, 9920 + p), inputs.sparse(p, n // 2, 9930 + p)])
+    want = oracle.heights(p, f)
+    t = dev_tensor(f)
+    for budget in (0, 8 << 20):
+        got = qfs.heights(p, t, form=form, power="identity", workspace_budget=budget).cpu().numpy()
+        assert np.array_equal(got, want), budget
+    assert qfs.read_status() == 0
+
+
+@pytest.mark.parametrize("p,power", [(5, "chain"), (7, "identity")])
+def test_classes_first_needed_in_a_capture(qfs, p, power):
+    # the workspace is prepared, the classes' buffer is not there yet: the first call is a captured one
+    f = inputs.dense(p, 300, 9940 + p)
+    t = dev_tensor(f)
+    out = torch.empty(300, dtype=torch.int8, device="cuda:0")
+    qfs.shutdown()
+    qfs.plan_prepare(7, 300)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        qfs.heights(p, t, out=out, power=power)
+    g.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(out.cpu().numpy(), oracle.heights(p, f))
+
+
 # ------------------------------------------------------------------------------------- edge cases and errors
 def test_edge_cases(qfs):
     p = 5
