@@ -542,6 +542,24 @@ def test_reduced_mode_heights(qfs, p, n):
     assert qfs.read_status() == 0
 
 
+@pytest.mark.parametrize("p,n", [(3, 1), (3, 2000), (5, 1), (5, 2000), (7, 1), (7, 700)])
+def test_reduced_kernel_and_general_route(qfs, p, n):
+    # one prime <= 7 takes the kernel of its own; a cap on the CTAs, or another prime, the fused launch
+    f = np.concatenate([inputs.dense(p, n, 9950 + p), inputs.sparse(p, n, 9960 + p)])
+    f[n // 2, 3] = p
+    want = oracle.heights(p, f)
+    assert want[n // 2] == -1
+    t = dev_tensor(f)
+    for kw in ({}, {"max_ctas": 5}):
+        assert np.array_equal(qfs.heights(p, t, power="reduced", **kw).cpu().numpy(), want), kw
+    other = 5 if p == 7 else 7
+    f2 = inputs.sparse(other, 40, 9970)
+    for q, g in ((p, f[n:]), (other, f2)):
+        got = qfs.heights_multi([(p, t, None), (q, dev_tensor(g), None)], power="reduced")
+        assert np.array_equal(got[0].cpu().numpy(), want)
+        assert np.array_equal(got[1].cpu().numpy(), oracle.heights(q, g))
+
+
 def test_reduced_mode_paper_examples(qfs):
     for p in (5, 7, 11, 13):
         sel = [r for r in example_quartics() if r[0] == p]
@@ -699,6 +717,17 @@ def test_poly_power_paper_workload_evaluation(qfs, n):
     mod = (1 << 127) - 1
     pt = (3, 5, 7, 11)
     assert _eval_mod(P, 16 * n, pt, mod) == pow(_eval_mod(f, 16, pt, mod), n, mod)
+
+
+def test_poly_power_primes_in_groups(qfs):
+    # five primes whose transforms of 2^23 words run two at a time, the last one alone
+    rng = np.random.default_rng(28)
+    f = [int(x) for x in rng.integers(0, 5, len(oracle.form_monomials(16)))]
+    f[0] = 4
+    P = qfs.poly_power(16, f, 12)
+    mod = (1 << 127) - 1
+    pt = (2, 3, 13, 17)
+    assert _eval_mod(P, 16 * 12, pt, mod) == pow(_eval_mod(f, 16, pt, mod), 12, mod)
 
 
 def test_poly_power_errors(qfs):
