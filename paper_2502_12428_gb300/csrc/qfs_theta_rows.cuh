@@ -9,7 +9,7 @@
 // of theta_poly takes a scatter of every class into the cube, a barrier per class and a byte load per MAC.)
 //
 // Bound by instruction issue.  Whole calls, by cube and by rows: p = 5, 131,071 sparse quartics (4.4 steps each) 133.9 and
-// 116.2 ms; p = 5, 65,536 dense 25.1 and 24.2 ms; 65 quartics at p = 3, where up to ten steps follow each other, 93 and 66 us.
+// 105.8 ms; p = 5, 65,536 dense 25.1 and 21.9 ms; 65 quartics at p = 3, where up to ten steps follow each other, 93 and 66 us.
 // The identity mode at p = 7, 65,536 dense quartics (9,400 past height 1): 41.8 and 23.7 ms.
 #pragma once
 #include <cstdint>
@@ -85,37 +85,53 @@ __device__ __forceinline__ void row_class_tables(uint32_t *ring) {
 }
 
 // Padded Delta (degree D) -> the classes `rc`; class s2 + p s3 + p^2 s4 holds Delta[p e + sigma], sigma = (.., s2, s3, s4)
-// per exponent.  Also builds the tables of theta_rows.  Ends with a barrier.
+// per exponent.  A warp takes every eighth class and gathers it word by word, kAhead words per lane at a time to have as
+// many loads in flight; the reads of a row's bytes meet in L1 and the stores are whole rows.  (A scatter of Delta's
+// bytes, chunk by chunk, writes a sector per byte: at p = 5, 92,000 of them per quartic, 115.9 ms per 131,071 sparse
+// quartics against 105.8, and 24.3 ms per 65,536 dense ones against 21.9.)  Also builds the tables of theta_rows.  Ends
+// with a barrier.
 template <int P>
-__device__ __noinline__ void delta_to_rows(const uint32_t *__restrict__ delta, uint32_t *__restrict__ rc, const Smem &sm,
+__device__ __noinline__ void delta_to_rows(const uint32_t *delta, uint32_t *__restrict__ rc, const Smem &sm,
                                            uint32_t *ring) {
   using Q = RowClasses<P>;
-  constexpr int D = Prime<P>::D;
-  const int *slice = reinterpret_cast<const int *>(ring + Q::o_slice);
-  for (int i = threadIdx.x; i < Q::n_cls * Q::words / 4; i += blockDim.x)
-    reinterpret_cast<uint4 *>(rc)[i] = make_uint4(0u, 0u, 0u, 0u);
+  constexpr int kAhead = 5;
   row_class_tables<P>(ring);
   __syncthreads();
-  uint8_t *rb = reinterpret_cast<uint8_t *>(rc);
-  const int nchunks = sm.SW[D + 1] / 4;
-  for (int k = threadIdx.x; k < nchunks; k += blockDim.x) {
-    int U, S, c;
-    decode_form_chunk(k, D, sm.SW, U, S, c);
-    const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(delta + 4 * k));   // a crew's write
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    const int e2 = U - S, q2 = e2 / P, r2 = e2 - P * q2;
-    const int T0 = 16 * c;
-    int q4 = T0 / P, r4 = T0 - P * q4;                 // e4 = T
-    int q3 = (S - T0) / P, r3 = (S - T0) - P * q3;     // e3 = S - T (>= 0 while T <= S)
+  const uint16_t *items = reinterpret_cast<const uint16_t *>(ring + Q::o_items);
+  const int *slice = reinterpret_cast<const int *>(ring + Q::o_slice);
+  const uint8_t *db = reinterpret_cast<const uint8_t *>(delta);
+  const int lane = threadIdx.x & 31;
+  for (int x = threadIdx.x >> 5; x < Q::n_cls; x += kThreads / 32) {
+    int r2, r3, r4;
+    const int k = class_kernel<P>(x, r2, r3, r4);
+    const int s3 = P - 1 - r3, s4 = P - 1 - r4, su = 3 * (P - 1) - r2 - r3 - r4;   // sigma
+    uint32_t *out = rc + (size_t)x * Q::words;
+    for (int i = lane; i < Q::zero; i += 32) out[i] = 0;
+    for (int i0 = 0; i0 < Q::n_items; i0 += 32 * kAhead) {
+      uint32_t v[kAhead];
+      int at[kAhead];
+      bool first[kAhead];
 #pragma unroll
-    for (int b = 0; b < 16; ++b) {
-      if (T0 + b <= S) {
-        const int up = q2 + q3 + q4, sp = q3 + q4;
-        rb[4 * ((r2 + P * r3 + P * P * r4) * Q::words + class_row<P>(slice, up, sp) + 1) + q4] =
-            (uint8_t)(w[b >> 2] >> (8 * (b & 3)));
+      for (int j = 0; j < kAhead; ++j) {
+        const int i = i0 + 32 * j + lane;
+        int u = 0, s = 0, w = 0;
+        if (i < Q::n_items) rows::item_of(items, i, u, s, w);
+        at[j] = i < Q::n_items ? class_row<P>(slice, u, s) + w : -1;
+        first[j] = w == 0;
+        v[j] = 0;
+        if (i < Q::n_items && u <= Q::d - k) {
+          const uint8_t *q = db + 4 * (sm.SW[P * u + su] + colw(P * s + s3 + s4)) + 4 * P * w + s4;
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            if (4 * w + r <= s) v[j] |= (uint32_t)q[P * r] << (8 * r);
+        }
       }
-      if (++r4 == P) { r4 = 0; ++q4; }
-      if (--r3 < 0) { r3 = P - 1; --q3; }
+#pragma unroll
+      for (int j = 0; j < kAhead; ++j)
+        if (at[j] >= 0) {
+          if (first[j]) out[at[j]] = 0;
+          out[at[j] + 1] = v[j];
+        }
     }
   }
   __syncthreads();
