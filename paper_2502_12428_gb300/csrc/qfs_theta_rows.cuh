@@ -9,7 +9,7 @@
 // of theta_poly takes a scatter of every class into the cube, a barrier per class and a byte load per MAC.)
 //
 // Bound by instruction issue.  Whole calls, by cube and by rows: p = 5, 131,071 sparse quartics (4.4 steps each) 133.9 and
-// 105.8 ms; p = 5, 65,536 dense 25.1 and 21.9 ms; 65 quartics at p = 3, where up to ten steps follow each other, 93 and 66 us.
+// 102.4 ms; p = 5, 65,536 dense 25.1 and 21.6 ms; 65 quartics at p = 3, where up to ten steps follow each other, 93 and 66 us.
 // The identity mode at p = 7, 65,536 dense quartics (9,400 past height 1): 41.8 and 23.7 ms.
 #pragma once
 #include <cstdint>
@@ -27,7 +27,7 @@ struct RowClasses {
   static constexpr int round = kThreads / kQuarters, items = (n_items + round - 1) / round * round;
   static constexpr int words = (zero + n_items + tri(d + 1) + 3) & ~3;           // of a class
   static constexpr int units = kQuarters * items / kThreads;                     // (output word, quarter) per thread
-  static constexpr int group = P == 3 ? n_cls + 1 : P == 5 ? 8 : 4;              // classes staged at a time
+  static constexpr int group = P == 3 ? n_cls + 1 : P == 5 ? 12 : 4;             // classes staged at a time
   static constexpr int groups = (n_cls + group - 1) / group;
   static constexpr int slots = groups > 1 ? 2 : 1;
   // shared memory, word offsets
