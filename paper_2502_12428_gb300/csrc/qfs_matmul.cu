@@ -17,11 +17,13 @@
 // What bounds it: the copies from L2 into shared memory (48 KB per K step of a tile, 512 clocks of MMAs: more than the
 // 64 bytes per clock and SM that L2 delivers), a last wave of tiles, and about 20 us of packing at n = 5,000.  n = m =
 // k, mod 11: 132 us at 5,000 and 773 us at 10,000 (1.90 and 2.59 PFLOP/s with the pack), against 1,895 us and 13.9 ms
-// by mma.sync m16n8k32 u8, which ran at 0.82 and 0.91 of its own peak; mod 101 and 251 at 5,000: 347 and 360 us.  At
-// 64 x 64 x 64 a call takes 15 us.
+// by mma.sync m16n8k32 u8, which ran at 0.82 and 0.91 of its own peak; mod 101 and 251 at 5,000: 347 and 360 us.  Up
+// to about 512 x 512 x 512 a call takes as long as the host needs to enqueue it (17 to 20 us).  The product kernel
+// starts while the pack runs (programmatic dependent launch): 700 x 90 x 3,000 mod 31 took 32.9 us, takes 28.8.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 
 #include "qfs_common.cuh"
@@ -77,6 +79,7 @@ __global__ void __launch_bounds__(256) pack_kernel(const uint8_t *__restrict__ A
   __shared__ uint8_t lut[PLANES][256];
   __shared__ __align__(16) uint32_t t[PLANES][kPackTile][kPackTile / 4 + 1];
   const int tid = threadIdx.x;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the product's CTAs set themselves up meanwhile
   {
     int v = tid % p;
     if (2 * v > p) v -= p;
@@ -233,6 +236,7 @@ __global__ void __launch_bounds__(kMMThreads, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the planes are packed, and whatever read C is done
   const int tiles_n = (n + kBM - 1) / kBM, tiles = tiles_n * ((m + kBN - 1) / kBN);
 
   if (warp == 0) {
@@ -406,11 +410,13 @@ cudaError_t launch(int p, int n, int m, int k, const uint8_t *A, const uint8_t *
   uint8_t *Ap = scratch, *Bp = scratch + plane_stride(n, kp, PLANES);
   Maps maps;
   if (!encoder()) return cudaErrorNotSupported;
-  for (int pl = 0; pl < 2; ++pl) {
-    const int q = pl < PLANES ? pl : 0;
-    if (!plane_map(&maps.a[pl], Ap + (size_t)q * n * kp, n, kp, kBM) ||
-        !plane_map(&maps.b[pl], Bp + (size_t)q * m * kp, m, kp, kBN))
+  for (int pl = 0; pl < PLANES; ++pl)
+    if (!plane_map(&maps.a[pl], Ap + (size_t)pl * n * kp, n, kp, kBM) ||
+        !plane_map(&maps.b[pl], Bp + (size_t)pl * m * kp, m, kp, kBN))
       return cudaErrorInvalidValue;
+  if (PLANES == 1) {   // (not read)
+    maps.a[1] = maps.a[0];
+    maps.b[1] = maps.b[0];
   }
   const dim3 pgrid(kp / kPackTile, (unsigned)((n > m ? n : m) + kPackTile - 1) / kPackTile, 2);
   pack_kernel<PLANES><<<pgrid, 256, 0, st>>>(A, B, n, m, k, kp, p, Ap, Bp);
@@ -424,13 +430,30 @@ cudaError_t launch(int p, int n, int m, int k, const uint8_t *A, const uint8_t *
   const uint32_t bias = (uint32_t)(((1 << 24) + p - 1) / p * p);
   const uintptr_t al = reinterpret_cast<uintptr_t>(C) | (uintptr_t)m;
   const int vec = (al & 15) == 0 ? 16 : (al & 7) == 0 ? 8 : (al & 3) == 0 ? 4 : 1;
-  e = cudaFuncSetAttribute(product_kernel<PLANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mm_smem(PLANES));
-  if (e != cudaSuccess) return e;
+  // the attribute is set once per device: a small product takes as long as the host needs to enqueue it (17 us)
+  static std::atomic<uint64_t> attribute_set{0};
+  int dev = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  const uint64_t bit = 1ull << (dev & 63);
+  if (!(attribute_set.load() & bit)) {
+    e = cudaFuncSetAttribute(product_kernel<PLANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mm_smem(PLANES));
+    if (e != cudaSuccess) return e;
+    attribute_set.fetch_or(bit);
+  }
   const long long tiles = (long long)((n + kBM - 1) / kBM) * ((m + kBN - 1) / kBN);
   const int grid = (int)(tiles < sms ? tiles : sms);
-  product_kernel<PLANES><<<grid, kMMThreads, mm_smem(PLANES), st>>>(maps, C, n, m, kp / kBK, (int)chunk, p, magic, bias,
-                                                                    vec, status);
-  return cudaGetLastError();
+  // The product may start while the pack runs; it waits for it after setting up its barriers and TMEM.
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute early;
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kMMThreads);
+  cfg.dynamicSmemBytes = mm_smem(PLANES);
+  cfg.stream = st;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, product_kernel<PLANES>, maps, C, n, m, kp / kBK, (int)chunk, p, magic, bias, vec, status);
 }
 
 }  // namespace
