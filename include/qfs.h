@@ -24,7 +24,8 @@
  *   - Errors that can be seen on the host are returned synchronously and nothing is enqueued.  n = 0 is a no-op.
  *   - The library owns its workspaces (one set per device, grown on demand, freed by qfs_shutdown).  Growing a
  *     workspace calls cudaMalloc; call qfs_plan_prepare for the largest p and batch first when capturing the
- *     calls into a CUDA graph.
+ *     calls into a CUDA graph.  The buffer of theta's residue classes (fused engine; p <= 5, and p = 7 in the identity
+ *     mode; at most 0.5 GB) has one size per prime and is allocated at its first use, which may be a captured call.
  *   - Calls are not thread-safe with respect to each other on the same device.
  */
 #ifndef QFS_H
@@ -98,8 +99,10 @@ typedef struct {
 
 /* Heights of n quartics over F_p.  coeffs: device, n x 35 uint8.  heights_out: device, n int8.
    Returns QFS_OK or an error status (nothing enqueued on error).
-   The fused engine enqueues two kernels: a height-1 screen (Fedder's criterion, one warp per quartic), which writes
-   1 or -1 for the rows it settles and lists the others, then the persistent launch over the listed rows. */
+   The fused engine enqueues a height-1 screen (Fedder's criterion, one warp per quartic), which writes 1 or -1 for the
+   rows it settles and lists the others, then the persistent launch over the listed rows.  A small batch at p >= 7
+   enqueues the launch once per number of CTAs that may share a quartic (1, 2, 4, 8); the number of listed rows
+   decides on the device which one runs. */
 int qfs_heights(int p, int64_t n, const uint8_t *coeffs, int max_h, int8_t *heights_out, cudaStream_t stream);
 
 /* Several batches, possibly over different primes, in one persistent launch (groups is a host array of
