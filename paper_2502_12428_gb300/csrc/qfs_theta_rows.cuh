@@ -3,7 +3,7 @@
 // theta(g) = sum_sigma Delta_sigma * g_rho over the p^3 residue classes (qfs_engine.cuh, Poly): products of forms whose
 // kernel g_rho has degree k <= 3.  Delta is split once per quartic (the identity mode forms it class by class) into one array
 // per class, all of one size, in global memory: rows (u, s) of bytes, each after a zero word (rows beyond the class's degree are zero), behind a zero row.  A
-// step copies the classes through shared memory by cp.async, kGroup at a time (all of them at p = 3), one barrier per
+// step copies the classes through shared memory by cp.async, a group at a time (all of them at p = 3), one barrier per
 // group, and multiplies them as they lie there: a thread takes one output word (four outputs) and every fourth class
 // (p = 7: four output words and every class), reads two words of each input row and meets the taps by dp4a in the windows of qfs_block.cuh.  (The padded byte cube
 // of theta_poly takes a scatter of every class into the cube, a barrier per class and a byte load per MAC.)

@@ -248,6 +248,24 @@ def test_theta_matrix_by_crews_repeats(qfs):
     assert qfs.read_status() == 0
 
 
+@pytest.mark.parametrize("p,n,m,k", [(11, 70, 300, 513), (251, 130, 257, 129)])
+def test_matmul_mod_captured(qfs, p, n, m, k):
+    # the product starts while the pack runs, also when replayed: every replay sees the operands of that moment
+    rng = np.random.default_rng(p)
+    A, B = (dev_tensor(rng.integers(0, p, s).astype(np.uint8)) for s in ((n, k), (k, m)))
+    out = qfs.matmul_mod(p, A, B)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        qfs.matmul_mod(p, A, B, out=out)
+    for _ in range(3):
+        A.copy_(dev_tensor(rng.integers(0, p, (n, k)).astype(np.uint8)))
+        g.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(out.cpu().numpy(), oracle.matmul_mod(p, A.cpu().numpy(), B.cpu().numpy()))
+    assert qfs.read_status() == 0
+
+
 # ------------------------------------------------------------------------------------- theta by rows
 @pytest.mark.parametrize("p,n", [(3, 4000), (5, 6000)])
 @pytest.mark.parametrize("form", CORE_FORMS)
