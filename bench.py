@@ -170,8 +170,8 @@ class ClockSampler:
 
 # ----------------------------------------------------------------------------------------------- helpers
 # the sources the fused dp4a kernel is compiled from (its launch shape comes from qfs_api.cu's occupancy query)
-FUSED_KERNEL_SOURCES = ("qfs_layout.cuh", "qfs_common.cuh", "qfs_sweep.cuh", "qfs_engine.cuh", "qfs_kernels.cuh",
-                        "qfs_form_dp4a.cu")
+FUSED_KERNEL_SOURCES = ("qfs_layout.cuh", "qfs_common.cuh", "qfs_sweep.cuh", "qfs_block.cuh", "qfs_rows.cuh",
+                        "qfs_theta_rows.cuh", "qfs_engine.cuh", "qfs_kernels.cuh", "qfs_form_dp4a.cu")
 
 
 def kernel_source_hash():
