@@ -136,12 +136,15 @@ int ensure_list(DeviceState &S, size_t bytes) {
 // graphs never lose it; null if the memory is not there.  The first call may come during a stream capture whose
 // workspace was prepared, so the allocation is made in relaxed mode, which a capture allows.
 int64_t class_ctas(const DeviceState &S, int p) { return (int64_t)S.sms * (p == 7 ? 2 : 4); }
+size_t class_bytes(const DeviceState &S, int p) {
+  return row_class_words(p) * sizeof(uint32_t) * (size_t)class_ctas(S, p);
+}
 uint32_t *ensure_classes(DeviceState &S, int p) {
   void *&c = S.classes[(p - 3) / 2];
   if (!c) {
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
-    if (cudaMalloc(&c, row_class_words(p) * sizeof(uint32_t) * (size_t)class_ctas(S, p)) != cudaSuccess) {
+    if (cudaMalloc(&c, class_bytes(S, p)) != cudaSuccess) {
       c = nullptr;
       (void)cudaGetLastError();
     }
@@ -438,14 +441,14 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
   prm.stats = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(S->ctrl) + 16);
   prm.ws = reinterpret_cast<uint32_t *>(S->ws);
   prm.ws_words = plan.ws_words;
-  // theta by rows, unless the budget does not cover the classes as well; without them it runs by cubes
+  // theta by rows, unless the budget does not cover the classes' buffer as well (all of it, however few CTAs this launch
+  // has: that is what a first call allocates); without it theta runs by cubes
   int class_p = 0;
   for (int i = 0; i < prm.n_groups; ++i)
     if (theta_by_rows(prm.g[i].p, power)) class_p = std::max(class_p, prm.g[i].p);
   if (class_p && plan.ctas <= class_ctas(*S, class_p)) {
-    const size_t bytes = row_class_words(class_p) * sizeof(uint32_t) * (size_t)plan.ctas;
     const size_t budget = opts && opts->workspace_budget ? opts->workspace_budget : default_budget(*S);
-    if (bytes + workspace_words(plan.ctas, plan.ws_words) * sizeof(uint32_t) <= budget) {
+    if (class_bytes(*S, class_p) + workspace_words(plan.ctas, plan.ws_words) * sizeof(uint32_t) <= budget) {
       prm.classes = ensure_classes(*S, class_p);
       prm.class_words = row_class_words(class_p);
     }

@@ -1,0 +1,52 @@
+"""The host runtime (qfs_api.cu) over a fake device: what a call allocates and launches, without a GPU.
+
+tests/host_runtime.cu compiles the runtime with counting stand-ins for the CUDA calls and recorders for the kernel
+launchers, and prints one JSON line per scenario.
+"""
+import json
+import os
+import re
+import subprocess
+
+import pytest
+
+from test_layout_host import CSRC, ROOT, _nvcc
+
+MB = 1 << 20
+CONTROL_BYTES = 1024   # the control block and the rounding of small buffers
+
+
+@pytest.fixture(scope="module")
+def runtime(tmp_path_factory):
+    nvcc = _nvcc()
+    if not nvcc:
+        pytest.skip("nvcc not found")
+    exe = str(tmp_path_factory.mktemp("runtime") / "host_runtime")
+    subprocess.run([nvcc, "-gencode", "arch=compute_103a,code=sm_103a", "-std=c++17", "-I", CSRC,
+                    "-I", os.path.join(ROOT, "include"), os.path.join(ROOT, "tests", "host_runtime.cu"), "-o", exe],
+                   check=True, capture_output=True)
+
+    def run(**kw):
+        arg = ",".join(f"{k}={v}" for k, v in kw.items())
+        out = subprocess.run([exe, arg], check=True, capture_output=True, text=True).stdout
+        r = json.loads(out)
+        r["fused"] = [{k: int(v) for k, v in re.findall(r"(\w+)=(\d+)", x)} for x in r["launches"]
+                      if x.startswith("fused")]
+        return r
+    return run
+
+
+@pytest.mark.parametrize("p,power,n,budget", [(7, 1, 1, 8 * MB), (7, 1, 2, 8 * MB), (7, 1, 600, 8 * MB),
+                                              (7, 1, 100000, 1024 * MB), (7, 1, 100, 550 * MB), (5, 0, 4, 4 * MB),
+                                              (5, 0, 1000, 200 * MB), (3, 0, 2, 1 * MB), (3, 1, 500, 6 * MB)])
+@pytest.mark.parametrize("form", [0, 1, 2])
+def test_workspace_stays_within_the_budget(runtime, p, power, n, budget, form):
+    # everything but the list of screened rows (8 bytes each) counts: chain buffers and theta's classes
+    r = runtime(op="heights", p1=p, n1=n, power=power, budget=budget, form=form)
+    assert r["rc"] == 0 and len(r["fused"]) == 1
+    assert r["peak"] <= budget + 8 * n + CONTROL_BYTES
+
+
+@pytest.mark.parametrize("p,power", [(3, 0), (5, 0), (3, 1), (5, 1), (7, 1)])
+def test_default_budget_takes_theta_by_rows(runtime, p, power):
+    assert runtime(op="heights", p1=p, n1=100000, power=power)["fused"][0]["classes"] == 1
