@@ -417,40 +417,39 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
   prm.power_mode = power;
   if (engine == QFS_ENGINE_STAGED) return run_staged(*S, prm, opts, stream);
 
-  // the reduced mode of one small prime (dp4a form) has a kernel of its own, which needs no workspace; a call that caps
-  // the CTAs or mixes primes takes the fused kernel
-  int reduced_p = 0;
-  if (power == QFS_POWER_REDUCED && form == QFS_FORM_DP4A && max_p <= kReducedMaxP &&
-      !(opts && (opts->ctas_per_sm > 0 || opts->max_ctas > 0))) {
-    reduced_p = same_prime(prm) ? max_p : 0;
-  }
-  // shared memory: the largest iterate pair of the launch plus the largest ring any group's tile needs
-  int ring_words = 0;
-  for (int i = 0; i < prm.n_groups; ++i)
-    ring_words = std::max(ring_words, ring_words_for(prm.g[i].p, tile_for(prm.g[i].p),
-                                                     uses_ring_chain(form, prm.g[i].p), power));
-  const size_t smem = ring_offset_for(tet(4 * (max_p - 1) + 1)) + 4 * (size_t)ring_words;
-  Plan plan;
-  const bool one_prime = same_prime(prm);
-  rc = make_plan(*S, form, max_p, n_items, opts, plan, smem,
-                 form == QFS_FORM_DP4A && power == QFS_POWER_CHAIN ? &prm : nullptr);
-  if (rc) return rc;
   auto *n_list = reinterpret_cast<unsigned long long *>(static_cast<char *>(S->ctrl) + 32);
   prm.counter = n_list + 1;
   prm.status = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(S->ctrl) + 8);
   prm.stats = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(S->ctrl) + 16);
-  prm.ws = reinterpret_cast<uint32_t *>(S->ws);
-  prm.ws_words = plan.ws_words;
-  // theta by rows, unless the budget does not cover the classes' buffer as well (all of it, however few CTAs this launch
-  // has: that is what a first call allocates); without it theta runs by cubes
-  int class_p = 0;
-  for (int i = 0; i < prm.n_groups; ++i)
-    if (theta_by_rows(prm.g[i].p, power)) class_p = std::max(class_p, prm.g[i].p);
-  if (class_p && plan.ctas <= class_ctas(*S, class_p)) {
-    const size_t budget = opts && opts->workspace_budget ? opts->workspace_budget : default_budget(*S);
-    if (class_bytes(*S, class_p) + workspace_words(plan.ctas, plan.ws_words) * sizeof(uint32_t) <= budget) {
-      prm.classes = ensure_classes(*S, class_p);
-      prm.class_words = row_class_words(class_p);
+  const bool one_prime = same_prime(prm);
+  // the reduced mode of one small prime (dp4a form) has a kernel of its own, which needs no workspace (so no budget is
+  // too small for it); a call that caps the CTAs or mixes primes takes the fused kernel
+  const bool reduced = power == QFS_POWER_REDUCED && form == QFS_FORM_DP4A && max_p <= kReducedMaxP && one_prime &&
+                       !(opts && (opts->ctas_per_sm > 0 || opts->max_ctas > 0));
+  Plan plan;
+  if (!reduced) {
+    // shared memory: the largest iterate pair of the launch plus the largest ring any group's tile needs
+    int ring_words = 0;
+    for (int i = 0; i < prm.n_groups; ++i)
+      ring_words = std::max(ring_words, ring_words_for(prm.g[i].p, tile_for(prm.g[i].p),
+                                                       uses_ring_chain(form, prm.g[i].p), power));
+    const size_t smem = ring_offset_for(tet(4 * (max_p - 1) + 1)) + 4 * (size_t)ring_words;
+    rc = make_plan(*S, form, max_p, n_items, opts, plan, smem,
+                   form == QFS_FORM_DP4A && power == QFS_POWER_CHAIN ? &prm : nullptr);
+    if (rc) return rc;
+    prm.ws = reinterpret_cast<uint32_t *>(S->ws);
+    prm.ws_words = plan.ws_words;
+    // theta by rows, unless the budget does not cover the classes' buffer as well (all of it, however few CTAs this
+    // launch has: that is what a first call allocates); without it theta runs by cubes
+    int class_p = 0;
+    for (int i = 0; i < prm.n_groups; ++i)
+      if (theta_by_rows(prm.g[i].p, power)) class_p = std::max(class_p, prm.g[i].p);
+    if (class_p && plan.ctas <= class_ctas(*S, class_p)) {
+      const size_t budget = opts && opts->workspace_budget ? opts->workspace_budget : default_budget(*S);
+      if (class_bytes(*S, class_p) + workspace_words(plan.ctas, plan.ws_words) * sizeof(uint32_t) <= budget) {
+        prm.classes = ensure_classes(*S, class_p);
+        prm.class_words = row_class_words(class_p);
+      }
     }
   }
   // height-1 screen first: the persistent launch then runs only the quartics that pass it
@@ -463,7 +462,7 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
   if (e != cudaSuccess) return cuda_fail(e);
   prm.list = static_cast<const int64_t *>(S->list);
   prm.n_list = n_list;
-  if (reduced_p) return (e = reduced_launch(reduced_p, prm, S->sms, stream)) == cudaSuccess ? QFS_OK : cuda_fail(e);
+  if (reduced) return (e = reduced_launch(max_p, prm, S->sms, stream)) == cudaSuccess ? QFS_OK : cuda_fail(e);
   for (int i = 0; i < 4; ++i) prm.crews[i] = plan.crews[i];
   if (one_prime || std::max({plan.crews[1], plan.crews[2], plan.crews[3]}) == 0) prm.crews[0] = plan.grid;
   for (int i = 0; i < 4; ++i) {

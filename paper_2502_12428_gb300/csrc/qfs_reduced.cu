@@ -195,7 +195,7 @@ __device__ int reduced_quartic(const uint8_t *__restrict__ f35, int max_h, RSmem
   return 0;
 }
 
-// Persistent CTAs take the listed items of groups with prime P; the items of other primes are another launch's.
+// Persistent CTAs take the listed items; every group of the launch has prime P.
 template <int P>
 __global__ void __launch_bounds__(kRThreads) reduced_kernel(const __grid_constant__ FusedParams prm) {
   using Q = Red<P>;

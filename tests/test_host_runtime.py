@@ -50,3 +50,17 @@ def test_workspace_stays_within_the_budget(runtime, p, power, n, budget, form):
 @pytest.mark.parametrize("p,power", [(3, 0), (5, 0), (3, 1), (5, 1), (7, 1)])
 def test_default_budget_takes_theta_by_rows(runtime, p, power):
     assert runtime(op="heights", p1=p, n1=100000, power=power)["fused"][0]["classes"] == 1
+
+
+@pytest.mark.parametrize("p", [3, 5, 7])
+def test_reduced_kernel_takes_no_workspace(runtime, p):
+    # its forms live in shared memory: neither chain buffers nor classes, and no budget is too small
+    for budget in (0, 1):
+        r = runtime(op="heights", p1=p, n1=100000, p2=p, n2=7, power=2, budget=budget)
+        assert r["rc"] == 0 and r["launches"] == ["screen", "reduced"]
+        assert r["peak"] <= 8 * 100007 + CONTROL_BYTES
+    # the fused kernel's reduced mode needs a quartic's buffers
+    for kw in (dict(max_ctas=3), dict(p2=11, n2=1), dict(form=0)):
+        r = runtime(op="heights", p1=p, n1=1000, power=2, **kw)
+        assert r["rc"] == 0 and len(r["fused"]) == 1
+        assert runtime(op="heights", p1=p, n1=1000, power=2, budget=1, **kw)["rc"] == 5
