@@ -107,7 +107,8 @@ int qfs_heights(int p, int64_t n, const uint8_t *coeffs, int max_h, int8_t *heig
 
 /* Several batches, possibly over different primes, in one persistent launch (groups is a host array of
    n_groups <= QFS_MAX_GROUPS descriptors).  Work is ordered largest p first so the heaviest quartics start
-   early.  Same return convention as qfs_heights. */
+   early; clusters of CTAs take them together where the screen's counts say that it pays, single CTAs the rest.  Same
+   return convention as qfs_heights. */
 int qfs_heights_multi(int n_groups, const qfs_group_t *groups, int max_h, cudaStream_t stream);
 
 /* qfs_heights_multi with explicit options (opts may be NULL). */

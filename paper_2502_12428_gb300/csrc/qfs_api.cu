@@ -31,8 +31,8 @@ struct DeviceState {
   size_t total_mem = 0;
   void *ws = nullptr;          // persistent-CTA workspaces
   size_t ws_bytes = 0;
-  void *ctrl = nullptr;        // [8]: status (u32), [16]: stats (2 x u64); cleared by every fused launch: [32]: survivors,
-                               // [40]: work counter (u64 each)
+  void *ctrl = nullptr;        // [8]: status (u32), [16]: stats (2 x u64); cleared by every fused launch: [32]: work counters
+                               // (2 x u64), [48]: survivors of every group (QFS_MAX_GROUPS x u64)
   void *staged = nullptr;      // staged-engine survivor buffers
   size_t staged_bytes = 0;
   int *which = nullptr;        // theta-matrix export: which workspace buffer holds each quartic's Delta
@@ -46,6 +46,7 @@ struct DeviceState {
   size_t list_bytes = 0;
 };
 
+constexpr size_t kControlBytes = 48 + 8 * QFS_MAX_GROUPS;
 constexpr int kMaxDevices = 64;
 DeviceState g_dev[kMaxDevices];
 std::mutex g_mu;
@@ -86,9 +87,9 @@ int device_state(DeviceState **out) {
     S.sms = prop.multiProcessorCount;
     S.total_mem = prop.totalGlobalMem;
     S.supported = (prop.major == 10 && prop.minor == 3);
-    e = cudaMalloc(&S.ctrl, 64);
+    e = cudaMalloc(&S.ctrl, kControlBytes);
     if (e != cudaSuccess) return cuda_fail(e);
-    e = cudaMemset(S.ctrl, 0, 64);
+    e = cudaMemset(S.ctrl, 0, kControlBytes);
     if (e != cudaSuccess) return cuda_fail(e);
     S.init = true;
   }
@@ -255,24 +256,24 @@ bool form_supported(int form) { return form == QFS_FORM_INT32 || form == QFS_FOR
 // best use of the device while there are many; with few quartics past height 1, or with a few heavy ones (p = 11 beside
 // p = 5), CTAs run out of work while others are in the middle of a quartic.  1,001 random quartics at p = 7 take 5.4 ms
 // without crews and 3.2 ms with them, 48 theta matrices 3.1 and 2.2 ms, p = 5, 7 and 11 together (47 quartics
-// of p = 11 past height 1) 204 and 83 ms.
+// of p = 11 past height 1) 204 and 68 ms.
 //   One prime: the number of survivors decides on the device (crew_for).  A launch is made for each crew size that can
 // come up, and all but one find that it is not their turn.
-//   Several primes: one size, estimated here from the share 1/p of quartics past height 1 and the outputs of their
-// chains: the heaviest quartic should take at most half of what the launch takes if its work is spread evenly.
+//   Several primes: one launch, whose crews take the heavy quartics and then go on as single CTAs; which quartics those
+// are is decided on the device from the screen's counts (joint_items).  Only the crews' size is estimated here, from the
+// share 1/p of quartics past height 1: the heaviest quartic should take at most half of what the launch takes if its
+// work is spread evenly.
 bool same_prime(const FusedParams &prm) {
   for (int i = 1; i < prm.n_groups; ++i)
     if (prm.g[i].p != prm.g[0].p) return false;
   return true;
 }
 int mixed_crew(const FusedParams &prm, int slots) {
-  const int64_t outputs[kMaxP + 1] = {0, 0, 0, 20000, 0, 430000, 0, 8300000, 0, 0, 0, 400000000, 0, 1600000000};
   int64_t work = 0, heaviest = 0;
   for (int i = 0; i < prm.n_groups; ++i) {
     const int p = prm.g[i].p;
-    const int64_t rows = std::min<int64_t>(std::max<int64_t>(1, prm.g[i].n / p), 1 << 20);
-    work += outputs[p] * rows;
-    heaviest = std::max(heaviest, outputs[p]);
+    work += quartic_us(p) * std::min<int64_t>(std::max<int64_t>(1, prm.g[i].n / p), 1 << 20);
+    heaviest = std::max(heaviest, quartic_us(p));
   }
   const int64_t need = 2 * slots * heaviest / work;
   return need >= 8 ? 8 : need >= 4 ? 4 : need >= 2 ? 2 : 1;
@@ -417,8 +418,8 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
   prm.power_mode = power;
   if (engine == QFS_ENGINE_STAGED) return run_staged(*S, prm, opts, stream);
 
-  auto *n_list = reinterpret_cast<unsigned long long *>(static_cast<char *>(S->ctrl) + 32);
-  prm.counter = n_list + 1;
+  prm.counter = reinterpret_cast<unsigned long long *>(static_cast<char *>(S->ctrl) + 32);
+  unsigned long long *n_list = prm.counter + 2;
   prm.status = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(S->ctrl) + 8);
   prm.stats = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(S->ctrl) + 16);
   const bool one_prime = same_prime(prm);
@@ -455,7 +456,7 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
   // height-1 screen first: the persistent launch then runs only the quartics that pass it
   rc = ensure_list(*S, (size_t)n_items * sizeof(int64_t));
   if (rc) return rc;
-  cudaError_t e = cudaMemsetAsync(n_list, 0, 2 * sizeof(unsigned long long), stream);
+  cudaError_t e = cudaMemsetAsync(prm.counter, 0, (2 + QFS_MAX_GROUPS) * sizeof(unsigned long long), stream);
   if (e != cudaSuccess) return cuda_fail(e);
   const int64_t screen_ctas = std::min<int64_t>((n_items + 7) / 8, (int64_t)S->sms * 8);
   e = screen_launch(prm, max_p, static_cast<int64_t *>(S->list), n_list, (int)screen_ctas, stream);

@@ -1000,7 +1000,7 @@ __device__ __forceinline__ void delta_to_classes(const uint32_t *__restrict__ de
   for (int k = threadIdx.x; k < nchunks; k += blockDim.x) {
     int U, S, c;
     decode_form_chunk(k, D, sm.SW, U, S, c);
-    const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(delta + 4 * k));   // a crew's write
+    const uint4 v = *reinterpret_cast<const uint4 *>(delta + 4 * k);
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
     const int e2 = U - S, q2 = e2 / P, r2 = e2 - P * q2;
     const int T0 = 16 * c;
@@ -1591,7 +1591,7 @@ __device__ __noinline__ int reduced_height(Smem &sm, uint8_t *gs, uint8_t *gn, u
 }
 
 // Runs A1-A7 for one quartic with the CTA's two workspace buffers; returns the height code.  crewA: the first of the
-// crew's buffers if the CTA belongs to one (chain power mode, dp4a form), else null.  classes: row_class_words(p) words of
+// crew's buffers if the crew takes this quartic together (chain power mode, dp4a form, p >= 7), else null.  classes: row_class_words(p) words of
 // this CTA where theta_by_rows, or null.
 template <int P, int FORM, bool DEBUG>
 __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem &sm, uint8_t *gs, uint8_t *gn,
@@ -1607,8 +1607,7 @@ __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem 
   if (DEBUG)
     for (int i = tid; i < Pr::ld; i += blockDim.x) dbg.g[i] = gs[i];
   if (gs[Pr::witness] != 0) return 1;
-  uint32_t *own = bufA;   // a buffer that a crew leaves to this CTA, unless it is the first one
-  if constexpr (FORM == 1 && !DEBUG) {
+  if constexpr (FORM == 1 && !DEBUG && P >= 7) {
     // from here on the crew works in its first CTA's buffers
     if (crewA) {
       cur = cur == bufA ? crewA : crewA + (bufB - bufA);
@@ -1651,8 +1650,6 @@ __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem 
     } else if (by_rows) {
       if constexpr (P <= 5) delta_to_rows<P>(delta, classes, sm, ring);
     } else if (by_classes) {
-      // (theta by classes is not split: each CTA of a crew makes its own copy, in its own order of classes)
-      if (sm.rank != 0) dg = own;
       poly_tables<P>(ringb);
       delta_to_classes<P>(delta, dg, sm, ringb);
     }
@@ -1700,7 +1697,7 @@ struct FusedParams {
   int64_t n_items;
   int max_h;
   int sw_len;                         // SW entries to build (max D in this launch + 2)
-  unsigned long long *counter;        // work queue head (zeroed before launch)
+  unsigned long long *counter;        // work queue heads (zeroed before launch): [0] of the CTAs, [1] of the crews
   uint32_t *status;
   unsigned long long *stats;          // [0] quartics past the height-1 test, [1] theta steps run
   uint32_t *ws;                       // workspace: a guard, then 2 buffers of ws_words (the stride) per CTA
@@ -1708,11 +1705,27 @@ struct FusedParams {
   uint32_t *classes;                  // per CTA class_words words for theta by rows, or null
   size_t class_words;
   int crew;                           // CTAs per cluster of the launch (1: no clusters)
-  int crews[4];                       // crews of 2^i CTAs that run at once (0: no such launch is made); see crew_for
+  int crews[4];                       // crews of 2^i CTAs that run at once (0: no such launch is made); see crew_for.  A
+                                      // launch over several primes with crews is the only one: crews[0] is 0
   int power_mode;                     // 0: chain (Algorithm 1 literally), 1: identity shortcut, 2: reduced theta
-  const int64_t *list;                // if set: the items to run (the survivors of the height-1 screen) ...
-  const unsigned long long *n_list;   // ... and their count; if null, every item 0 .. n_items-1 runs
+  const int64_t *list;                // if set: the items to run (the survivors of the height-1 screen), every group's
+                                      // from its item_begin on ...
+  const unsigned long long *n_list;   // ... and their count for each group; if null, every item 0 .. n_items-1 runs
 };
+
+// Item k of those to run, group after group (the largest prime first).
+__device__ __forceinline__ int64_t listed_item(const FusedParams &prm, int64_t k) {
+  if (!prm.list) return k;
+  int g = 0;
+  for (; g + 1 < prm.n_groups && k >= (int64_t)prm.n_list[g]; ++g) k -= (int64_t)prm.n_list[g];
+  return prm.list[prm.g[g].item_begin + k];
+}
+__device__ __forceinline__ int64_t listed_items(const FusedParams &prm) {
+  if (!prm.list) return prm.n_items;
+  int64_t n = 0;
+  for (int g = 0; g < prm.n_groups; ++g) n += (int64_t)prm.n_list[g];
+  return n;
+}
 
 // The crew size for n_run quartics of one prime, among those that launches are made for.  Crews of 8 while each quartic
 // gets one at once, smaller ones for up to three rounds, as measured at p = 7 with random quartics of height >= 2 (ms per
@@ -1723,8 +1736,27 @@ __host__ __device__ inline int crew_for(int64_t n_run, const int (&crews)[4]) {
   if (n_run <= crews[3]) return 8;
   if (n_run <= 3 * (int64_t)crews[2]) return 4;
   if (n_run <= 3 * (int64_t)crews[1]) return 2;
-  if (crews[0] > 0) return 1;
-  return crews[1] > 0 ? 2 : crews[2] > 0 ? 4 : 8;   // several primes: the only one there is
+  return 1;
+}
+
+// Microseconds that a CTA takes for a quartic of prime p past height 1 (chain mode, dp4a form, random quartics) when
+// every SM has two of them to do.
+__host__ __device__ constexpr int64_t quartic_us(int p) {
+  return p == 3 ? 60 : p == 5 ? 500 : p == 7 ? 4500 : p == 11 ? 220000 : 800000;
+}
+
+// Several primes in one launch of `ctas` CTAs in crews: the leading items (n_list of them in each group, largest prime
+// first) that the crews take together; single CTAs take the rest.  The crews get a prime whose quartic takes one CTA
+// at least crew / 3 times as long as the whole launch takes with its work spread evenly; for a prime alone that is up to
+// three rounds of crews, as in crew_for.  At p <= 5 only the chain's products could be split, and single CTAs are always
+// better: 65,536 quartics at p = 5 take 21.6 ms by CTAs, 91 ms by crews of 8.
+__host__ __device__ inline int64_t joint_items(int n_groups, const FusedGroup *g, const unsigned long long *n_list,
+                                               int crew, int64_t ctas) {
+  int64_t work = 0, joint = 0;
+  for (int i = 0; i < n_groups; ++i) work += quartic_us(g[i].p) * (int64_t)n_list[i];
+  for (int i = 0; i < n_groups && g[i].p >= 7 && 3 * ctas * quartic_us(g[i].p) >= crew * work; ++i)
+    joint += (int64_t)n_list[i];
+  return joint;
 }
 
 // SMALL: an int8 tensor form launch whose primes are all <= 5; the kernel then needs no code for larger primes and
@@ -1732,8 +1764,16 @@ __host__ __device__ inline int crew_for(int64_t n_run, const int (&crews)[4]) {
 template <int FORM, bool SMALL>
 __device__ __forceinline__ void fused_body(const FusedParams &prm) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int64_t n_run = prm.list ? (int64_t)*prm.n_list : prm.n_items;
-  if (FORM == 1 && crew_for(n_run, prm.crews) != prm.crew) return;   // another launch's turn
+  const int64_t n_run = listed_items(prm);
+  int64_t n_joint = 0;   // items that the crews take together, before the rest
+  if constexpr (FORM == 1) {
+    if (prm.crews[0] == 0) {
+      n_joint = joint_items(prm.n_groups, prm.g, prm.n_list, prm.crew, gridDim.x);
+    } else {
+      if (crew_for(n_run, prm.crews) != prm.crew) return;   // another launch's turn
+      if (prm.crew > 1) n_joint = n_run;
+    }
+  }
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
   uint8_t *gs = smem_raw + sizeof(Smem);
   // the second iterate buffer follows the largest ld in this launch
@@ -1748,22 +1788,38 @@ __device__ __forceinline__ void fused_body(const FusedParams &prm) {
   DebugPtrs dbg{nullptr, nullptr, nullptr, nullptr};
   const int crew = FORM == 1 ? prm.crew : 1, rank = crew > 1 ? crew_rank() : 0;
   uint32_t *classes = prm.classes ? prm.classes + (size_t)blockIdx.x * prm.class_words : nullptr;
-  uint32_t *crewA = crew > 1 ? bufA - (size_t)rank * 2 * prm.ws_words : nullptr;
+  uint32_t *first = bufA - (size_t)rank * 2 * prm.ws_words;   // the crew's first buffer
+  bool joint = n_joint > 0;   // the crew works together; then each CTA for itself
+  // The first item of each crew (of each CTA, if no crew works together) is fixed by its place in the grid, so that few
+  // quartics go to those that were placed first, on SMs of their own: 15 quartics at p = 11 take 21 ms so, 26 ms by
+  // crews that share SMs.
+  const int64_t n_takers = joint ? gridDim.x / crew : gridDim.x;   // that have a fixed first item
+  int64_t take = joint ? blockIdx.x / crew : blockIdx.x;
+  const int64_t solo0 = joint ? n_joint : n_takers;   // first item that the CTAs' queue gives out
   for (;;) {
-    crew_sync(crew);
+    crew_sync(joint ? crew : 1);
     if (threadIdx.x == 0) {
       sm.crew = 1;   // until f^(p-1) is formed
       sm.rank = 0;
-      if (rank == 0) {
-        const int64_t k = (int64_t)atomicAdd(prm.counter, 1ull);
-        sm.item = k < n_run ? (prm.list ? prm.list[k] : k) : -1;
+      if (!joint) {
+        const int64_t k = take >= 0 ? take : solo0 + (int64_t)atomicAdd(prm.counter, 1ull);
+        sm.item = k < n_run ? listed_item(prm, k) : -1;
+      } else if (rank == 0) {
+        const int64_t k = take >= 0 ? take : n_takers + (int64_t)atomicAdd(prm.counter + 1, 1ull);
+        sm.item = k < n_joint ? listed_item(prm, k) : -1;
         for (int to = 1; to < crew; ++to)
           asm volatile("st.shared::cluster.s64 [%0], %1;" ::"r"(crew_addr(&sm.item, to)), "l"(sm.item) : "memory");
       }
     }
-    crew_sync(crew);
+    crew_sync(joint ? crew : 1);
+    take = -1;
     const int64_t item = sm.item;
-    if (item < 0) break;
+    if (item < 0) {
+      if (!joint) break;
+      joint = false;
+      continue;
+    }
+    uint32_t *crewA = joint ? first : nullptr;
     int gi = 0;
     while (gi + 1 < prm.n_groups && item >= prm.g[gi + 1].item_begin) ++gi;
     const FusedGroup &G = prm.g[gi];
@@ -1790,7 +1846,7 @@ __device__ __forceinline__ void fused_body(const FusedParams &prm) {
         }
         break;
     }
-    if (threadIdx.x == 0 && rank == 0) {
+    if (threadIdx.x == 0 && (!joint || rank == 0)) {
       G.heights[row] = (int8_t)h;
       if (h != 1 && h != -1) {
         atomicAdd(prm.stats, 1ull);

@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kScreenThreads) screen_kernel(const __grid_con
     }
     if (lane == 0) {
       if (r != 0) G.heights[row] = (int8_t)r;
-      else list[atomicAdd(n_list, 1ull)] = item;
+      else list[G.item_begin + (int64_t)atomicAdd(n_list + gi, 1ull)] = item;
     }
     __syncwarp();
   }

@@ -181,6 +181,15 @@ int main(int argc, char **argv) {
       o.workspace_budget = (size_t)num("budget", 0);
       o.max_ctas = (int)num("max_ctas", 0);
       rc = qfs_heights_multi_ex(n, g, 10, &o, nullptr);
+    } else if (op == "joint") {   // crews of a launch over several primes: survivors n1, n2, ... of groups p1 > p2 > ...
+      FusedGroup g[kMaxGroups] = {};
+      unsigned long long n_list[kMaxGroups] = {};
+      int n = 0;
+      for (; m.count("p" + std::to_string(n + 1)); ++n) {
+        g[n].p = (int)num(("p" + std::to_string(n + 1)).c_str(), 0);
+        n_list[n] = (unsigned long long)num(("n" + std::to_string(n + 1)).c_str(), 0);
+      }
+      rc = (int)joint_items(n, g, n_list, (int)num("crew", 8), num("ctas", 304));
     } else if (op == "prepare") {
       rc = qfs_plan_prepare((int)num("p", 7), num("n", 0));
     } else if (op == "theta_matrix") {

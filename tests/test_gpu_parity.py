@@ -248,6 +248,54 @@ def test_theta_matrix_by_crews_repeats(qfs):
     assert qfs.read_status() == 0
 
 
+def _ms(fn, reps=5):
+    """Milliseconds of fn() on the current stream, the least of `reps` passes after a first one."""
+    best = float("inf")
+    for i in range(reps + 1):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        fn()
+        b.record()
+        b.synchronize()
+        if i:
+            best = min(best, a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("p,n,big,past,limit", [(5, 30000, 11, False, 1.3), (5, 30000, 13, False, 1.3),
+                                                (3, 60000, 7, False, 1.3), (3, 60000, 7, True, 2.0)])
+def test_one_heavy_row_does_not_slow_a_mixed_launch(qfs, p, n, big, past, limit):
+    # many light quartics beside one row of a large prime: the crews serve that row only, and only if it is past height 1
+    # (then the launch takes as long as the row does on one CTA or a crew: 4.4 ms at most at p = 7, beside 3.5 ms)
+    f, _ = find_rows(big, 60, 9760 + big, lambda x: (x != 1) == past, 1)
+    light, heavy = dev_tensor(inputs.dense(p, n, 9750 + p)), dev_tensor(f)
+    out, out2 = (torch.empty(k, dtype=torch.int8, device="cuda:0") for k in (n, 1))
+    alone = _ms(lambda: qfs.heights(p, light, out=out))
+    want, want2 = out.clone(), qfs.heights(big, heavy)
+    mixed = _ms(lambda: qfs.heights_multi([(p, light, out), (big, heavy, out2)]))
+    assert torch.equal(out, want) and torch.equal(out2, want2)
+    assert mixed < limit * alone, (mixed, alone)
+    assert qfs.read_status() == 0
+
+
+@pytest.mark.parametrize("power", ["chain", "identity", "reduced"])
+def test_several_groups_of_several_primes(qfs, power):
+    # lists of survivors group by group: groups of one prime, empty ones, rows that are all height 1, invalid rows
+    groups = []
+    for p, n, gen in [(3, 900, inputs.sparse), (7, 40, inputs.dense), (5, 333, inputs.dense), (7, 1, inputs.sparse),
+                      (3, 1, inputs.dense), (11, 12, inputs.dense), (5, 70, inputs.sparse)]:
+        groups.append((p, gen(p, n, 9770 + n)))
+    groups[2][1][5, 0] = 5
+    groups.append((7, groups[1][1][oracle.heights(7, groups[1][1]) == 1]))
+    outs = qfs.heights_multi([(p, dev_tensor(f), None) for p, f in groups], power=power)
+    for (p, f), o in zip(groups, outs):
+        assert np.array_equal(o.cpu().numpy(), oracle.heights(p, f)), p
+    one = [g for g in groups if g[0] == 7]
+    for (p, f), o in zip(one, qfs.heights_multi([(p, dev_tensor(f), None) for p, f in one], power=power)):
+        assert np.array_equal(o.cpu().numpy(), oracle.heights(p, f))
+    assert qfs.read_status() == 0
+
+
 @pytest.mark.parametrize("p,n,m,k", [(11, 70, 300, 513), (251, 130, 257, 129)])
 def test_matmul_mod_captured(qfs, p, n, m, k):
     # the product starts while the pack runs, also when replayed: every replay sees the operands of that moment

@@ -64,3 +64,24 @@ def test_reduced_kernel_takes_no_workspace(runtime, p):
         r = runtime(op="heights", p1=p, n1=1000, power=2, **kw)
         assert r["rc"] == 0 and len(r["fused"]) == 1
         assert runtime(op="heights", p1=p, n1=1000, power=2, budget=1, **kw)["rc"] == 5
+
+
+@pytest.mark.parametrize("groups,crew,joint", [
+    (((11, 0), (5, 13000)), 8, 0),              # the one p = 11 row had height 1: every quartic by single CTAs
+    (((11, 1), (5, 13000)), 8, 1),              # it did not: a crew takes it, CTAs the rest
+    (((7, 1), (3, 8000)), 8, 1),
+    (((7, 1), (3, 20000)), 8, 0),               # the launch takes as long anyway
+    (((7, 0), (3, 20000)), 8, 0),
+    (((11, 47), (7, 2376), (5, 3440)), 4, 47),  # three primes: the crews take the largest
+    (((11, 1), (7, 9), (5, 13)), 8, 10),        # few quartics of any prime: those of p >= 7
+    (((11, 300), (5, 100)), 8, 0),              # many: one CTA each is the better split
+    (((13, 2), (11, 20)), 8, 22),
+])
+def test_crews_take_the_heavy_quartics_of_a_mixed_launch(runtime, groups, crew, joint):
+    kw = {f"{k}{i + 1}": v for i, g in enumerate(groups) for k, v in zip("pn", g)}
+    assert runtime(op="joint", crew=crew, ctas=304, **kw)["rc"] == joint
+
+
+def test_mixed_launch_is_one_launch(runtime):
+    r = runtime(op="heights", p1=5, n1=65536, p2=11, n2=1)
+    assert [f["crew"] for f in r["fused"]] == [8] and r["fused"][0]["grid"] == 304
