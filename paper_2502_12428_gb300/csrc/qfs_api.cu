@@ -282,6 +282,7 @@ int mixed_crew(const FusedParams &prm, int slots) {
 struct Plan {
   int grid = 0;        // CTAs of a launch without crews
   int crews[4] = {};   // crews of 2^i CTAs the device holds at once (0: not used)
+  int crew_rounds = 1; // see crew_for
   int64_t ctas = 0;    // CTAs that need buffers
   size_t smem = 0;
   size_t ws_words = 0;
@@ -301,7 +302,8 @@ int make_plan(DeviceState &S, int form, int max_p, int64_t n_items, const qfs_op
     const int tuned = sweep_for(form, max_p).ctas_per_sm;
     if (tuned > 0) per_sm = std::min(per_sm, tuned);
   }
-  int64_t grid = (int64_t)S.sms * per_sm;
+  const int64_t full = (int64_t)S.sms * per_sm;
+  int64_t grid = full;
   if (opts && opts->max_ctas > 0) grid = std::min<int64_t>(grid, opts->max_ctas);
   const size_t per_cta = 2 * plan.ws_words * sizeof(uint32_t);
   const size_t budget = opts && opts->workspace_budget ? opts->workspace_budget : default_budget(S);
@@ -309,7 +311,9 @@ int make_plan(DeviceState &S, int form, int max_p, int64_t n_items, const qfs_op
   int64_t ctas = std::min<int64_t>(grid, n_items);   // CTAs that need buffers
   if (prm && max_p >= 7 && !(opts && (opts->ctas_per_sm > 0 || opts->max_ctas > 0))) {
     const bool one_prime = same_prime(*prm);
-    const int want = one_prime ? 0 : mixed_crew(*prm, (int)grid);
+    int want = one_prime ? 0 : mixed_crew(*prm, (int)grid);
+    while (want > 1 && grid % want * 8 > grid) want /= 2;   // crews that would leave too much of a small grid unused
+    plan.crew_rounds = 4 * grid >= 3 * full ? 3 : 1;
     // a batch of one prime with many rows will not leave few survivors
     const bool few = one_prime && n_items / max_p <= 3 * grid;
     for (int i = 1; i < 4; ++i) {
@@ -465,6 +469,7 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
   prm.n_list = n_list;
   if (reduced) return (e = reduced_launch(max_p, prm, S->sms, stream)) == cudaSuccess ? QFS_OK : cuda_fail(e);
   for (int i = 0; i < 4; ++i) prm.crews[i] = plan.crews[i];
+  prm.crew_rounds = plan.crew_rounds;
   if (one_prime || std::max({plan.crews[1], plan.crews[2], plan.crews[3]}) == 0) prm.crews[0] = plan.grid;
   for (int i = 0; i < 4; ++i) {
     if (prm.crews[i] == 0) continue;

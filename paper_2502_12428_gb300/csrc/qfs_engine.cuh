@@ -1707,6 +1707,7 @@ struct FusedParams {
   int crew;                           // CTAs per cluster of the launch (1: no clusters)
   int crews[4];                       // crews of 2^i CTAs that run at once (0: no such launch is made); see crew_for.  A
                                       // launch over several primes with crews is the only one: crews[0] is 0
+  int crew_rounds;                    // quartics of one prime that a crew of 2 or more may take one after another
   int power_mode;                     // 0: chain (Algorithm 1 literally), 1: identity shortcut, 2: reduced theta
   const int64_t *list;                // if set: the items to run (the survivors of the height-1 screen), every group's
                                       // from its item_begin on ...
@@ -1732,10 +1733,13 @@ __device__ __forceinline__ int64_t listed_items(const FusedParams &prm) {
 // call by crews of 1, 2, 4 and 8; 304, 152, 76 and 38 run at once):
 //     36: 3.7, 2.1, 1.2, 1.0     100: 3.7, 2.8, 2.4, 2.7     160: 5.1, 4.1, 3.6, 4.1     250: 5.3, 5.2, 4.9, 6.0
 //     310: 7.0, 6.3, 6.1, 7.3    400: 8.0, 7.6, 7.6, 9.4     600: 10.4, 10.6, 11.4, 13.8
-__host__ __device__ inline int crew_for(int64_t n_run, const int (&crews)[4]) {
+// That is with two CTAs on every SM.  On a part of the device (a small workspace budget) a CTA has an SM to itself: one
+// quartic takes 2.8, 1.6, 1.0 and 0.6 ms, and crews are better only while each quartic gets one at once (`rounds` = 1; 3
+// quartics on 3 CTAs: 2.8 ms, by one crew of 2 4.7 ms).
+__host__ __device__ inline int crew_for(int64_t n_run, const int (&crews)[4], int rounds) {
   if (n_run <= crews[3]) return 8;
-  if (n_run <= 3 * (int64_t)crews[2]) return 4;
-  if (n_run <= 3 * (int64_t)crews[1]) return 2;
+  if (n_run <= rounds * (int64_t)crews[2]) return 4;
+  if (n_run <= rounds * (int64_t)crews[1]) return 2;
   return 1;
 }
 
@@ -1747,14 +1751,14 @@ __host__ __device__ constexpr int64_t quartic_us(int p) {
 
 // Several primes in one launch of `ctas` CTAs in crews: the leading items (n_list of them in each group, largest prime
 // first) that the crews take together; single CTAs take the rest.  The crews get a prime whose quartic takes one CTA
-// at least crew / 3 times as long as the whole launch takes with its work spread evenly; for a prime alone that is up to
-// three rounds of crews, as in crew_for.  At p <= 5 only the chain's products could be split, and single CTAs are always
+// at least crew / rounds times as long as the whole launch takes with its work spread evenly; for a prime alone that is up
+// to that many rounds of crews, as in crew_for.  At p <= 5 only the chain's products could be split, and single CTAs are always
 // better: 65,536 quartics at p = 5 take 21.6 ms by CTAs, 91 ms by crews of 8.
 __host__ __device__ inline int64_t joint_items(int n_groups, const FusedGroup *g, const unsigned long long *n_list,
-                                               int crew, int64_t ctas) {
+                                               int crew, int64_t ctas, int rounds) {
   int64_t work = 0, joint = 0;
   for (int i = 0; i < n_groups; ++i) work += quartic_us(g[i].p) * (int64_t)n_list[i];
-  for (int i = 0; i < n_groups && g[i].p >= 7 && 3 * ctas * quartic_us(g[i].p) >= crew * work; ++i)
+  for (int i = 0; i < n_groups && g[i].p >= 7 && rounds * ctas * quartic_us(g[i].p) >= crew * work; ++i)
     joint += (int64_t)n_list[i];
   return joint;
 }
@@ -1768,9 +1772,9 @@ __device__ __forceinline__ void fused_body(const FusedParams &prm) {
   int64_t n_joint = 0;   // items that the crews take together, before the rest
   if constexpr (FORM == 1) {
     if (prm.crews[0] == 0) {
-      n_joint = joint_items(prm.n_groups, prm.g, prm.n_list, prm.crew, gridDim.x);
+      n_joint = joint_items(prm.n_groups, prm.g, prm.n_list, prm.crew, gridDim.x, prm.crew_rounds);
     } else {
-      if (crew_for(n_run, prm.crews) != prm.crew) return;   // another launch's turn
+      if (crew_for(n_run, prm.crews, prm.crew_rounds) != prm.crew) return;   // another launch's turn
       if (prm.crew > 1) n_joint = n_run;
     }
   }

@@ -19,6 +19,7 @@ size_t limit = ~size_t(0), live = 0, peak = 0;
 std::map<uintptr_t, size_t> blocks;
 uintptr_t next = 1 << 20;
 std::vector<std::string> launches;
+int crews[4], rounds;   // of the last fused launch
 
 cudaError_t alloc(void **p, size_t n) {
   if (live + n > limit) return cudaErrorMemoryAllocation;
@@ -72,6 +73,8 @@ namespace qfs {
   template <>                                                                                                          \
   cudaError_t FormLauncher<F>::fused(const FusedParams &prm, int grid, size_t smem, cudaStream_t, bool) {              \
     fake::record("fused form=%d grid=%d crew=%d smem=%zu classes=%d", F, grid, prm.crew, smem, prm.classes != nullptr); \
+    for (int i = 0; i < 4; ++i) fake::crews[i] = prm.crews[i];                                                         \
+    fake::rounds = prm.crew_rounds;                                                                                    \
     return cudaSuccess;                                                                                                \
   }                                                                                                                    \
   template <>                                                                                                          \
@@ -189,13 +192,16 @@ int main(int argc, char **argv) {
         g[n].p = (int)num(("p" + std::to_string(n + 1)).c_str(), 0);
         n_list[n] = (unsigned long long)num(("n" + std::to_string(n + 1)).c_str(), 0);
       }
-      rc = (int)joint_items(n, g, n_list, (int)num("crew", 8), num("ctas", 304));
+      rc = (int)joint_items(n, g, n_list, (int)num("crew", 8), num("ctas", 304), 3);
     } else if (op == "prepare") {
       rc = qfs_plan_prepare((int)num("p", 7), num("n", 0));
     } else if (op == "theta_matrix") {
       rc = qfs_theta_matrix((int)num("p", 7), num("n", 1), rows, rows, nullptr);
     }
-    std::printf("{\"rc\": %d, \"live\": %zu, \"peak\": %zu, \"launches\": [", rc, fake::live, fake::peak);
+    std::printf("{\"crews\": [%d, %d, %d, %d], \"crew_for\": [", fake::crews[0], fake::crews[1], fake::crews[2],
+                fake::crews[3]);
+    for (int n = 0; n <= 700; ++n) std::printf("%s%d", n ? ", " : "", crew_for(n, fake::crews, fake::rounds));
+    std::printf("], \"rc\": %d, \"live\": %zu, \"peak\": %zu, \"launches\": [", rc, fake::live, fake::peak);
     for (size_t i = 0; i < fake::launches.size(); ++i) std::printf("%s\"%s\"", i ? ", " : "", fake::launches[i].c_str());
     std::printf("]}\n");
   }

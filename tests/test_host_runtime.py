@@ -85,3 +85,28 @@ def test_crews_take_the_heavy_quartics_of_a_mixed_launch(runtime, groups, crew, 
 def test_mixed_launch_is_one_launch(runtime):
     r = runtime(op="heights", p1=5, n1=65536, p2=11, n2=1)
     assert [f["crew"] for f in r["fused"]] == [8] and r["fused"][0]["grid"] == 304
+
+
+@pytest.mark.parametrize("p,cta_bytes", [(7, 2 * 245904 * 4), (11, 2 * 5052676 * 4)])
+def test_small_budgets_use_crews_only_while_each_quartic_gets_one(runtime, p, cta_bytes):
+    # a crew of c takes a quartic in more than 1/c of a CTA's time: a second round of crews on a small grid is slower than
+    # a CTA for each quartic (7 on a budget of 7 CTAs)
+    for ctas in (1, 2, 3, 4, 5, 7, 8, 13, 40, 152, 200):
+        r = runtime(op="heights", p1=p, n1=2 * ctas, budget=ctas * cta_bytes)
+        assert r["rc"] == 0 and r["crews"][0] == ctas
+        assert r["peak"] <= ctas * cta_bytes + 8000 + CONTROL_BYTES
+        for n, crew in enumerate(r["crew_for"][:2 * ctas + 1]):
+            assert n == 0 or crew == 1 or n <= r["crews"][crew.bit_length() - 1]
+            if 1 <= n <= ctas // 2:
+                assert crew > 1   # there is room for a crew of 2 for each
+    # the whole device: two CTAs per SM share it, and up to three rounds of crews are faster
+    r = runtime(op="heights", p1=p, n1=1000)
+    assert r["crews"] == [304, 152, 76, 38]
+    assert [r["crew_for"][n] for n in (1, 38, 39, 228, 229, 456, 457)] == [8, 8, 4, 4, 2, 2, 1]
+
+
+def test_mixed_launch_on_a_small_budget_uses_its_ctas(runtime):
+    for ctas in (1, 3, 7, 13, 40, 100):
+        r = runtime(op="heights", p1=5, n1=3000, p2=11, n2=30, budget=ctas * 2 * 5052676 * 4)
+        assert r["rc"] == 0 and len(r["fused"]) == 1
+        assert r["fused"][0]["grid"] >= ctas - ctas // 8
