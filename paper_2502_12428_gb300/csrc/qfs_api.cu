@@ -47,6 +47,7 @@ struct DeviceState {
 };
 
 constexpr size_t kControlBytes = 48 + 8 * QFS_MAX_GROUPS;
+constexpr int kMinRowBlock = 1024;   // rows of A that a mod-p product takes at least at once, whatever the memory
 constexpr int kMaxDevices = 64;
 DeviceState g_dev[kMaxDevices];
 std::mutex g_mu;
@@ -98,20 +99,26 @@ int device_state(DeviceState **out) {
   return QFS_OK;
 }
 
-int ensure_workspace(DeviceState &S, size_t bytes) {
+// A workspace of `bytes`.  enough: what the caller can do with; a workspace of that size stays where it is if there is no
+// memory for the larger one.
+int ensure_workspace(DeviceState &S, size_t bytes, size_t enough) {
   if (S.ws_bytes >= bytes) return QFS_OK;
+  void *bigger = nullptr;
+  if (S.ws && S.ws_bytes >= enough && cudaMalloc(&bigger, bytes) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return QFS_ERR_NO_MEMORY;
+  }
   if (S.ws) {
     cudaError_t e = cudaFree(S.ws);
     S.ws = nullptr;
     S.ws_bytes = 0;
     if (e != cudaSuccess) return cuda_fail(e);
   }
-  cudaError_t e = cudaMalloc(&S.ws, bytes);
-  if (e != cudaSuccess) {
-    S.ws = nullptr;
+  if (!bigger && cudaMalloc(&bigger, bytes) != cudaSuccess) {
     (void)cudaGetLastError();
     return QFS_ERR_NO_MEMORY;
   }
+  S.ws = bigger;
   S.ws_bytes = bytes;
   return QFS_OK;
 }
@@ -192,7 +199,8 @@ int run_staged(DeviceState &S, const FusedParams &prm, const qfs_options_t *opts
     grid = std::min<int64_t>(grid, (int64_t)(budget / 2 / per_cta));
     if (grid < 1) return QFS_ERR_NO_MEMORY;
     pl.grid = (int)grid;
-    int rc = ensure_workspace(S, workspace_words(grid, pl.ws_words) * sizeof(uint32_t));
+    const size_t ws_bytes = workspace_words(grid, pl.ws_words) * sizeof(uint32_t);
+    int rc = ensure_workspace(S, ws_bytes, ws_bytes);
     if (rc) return rc;
     const size_t per_surv = staged_survivor_bytes(p);
     int64_t chunk = std::min<int64_t>({g.n, (int64_t)8192, (int64_t)((budget / 2) / per_surv)});
@@ -330,7 +338,14 @@ int make_plan(DeviceState &S, int form, int max_p, int64_t n_items, const qfs_op
   if (grid < 1) return QFS_ERR_NO_MEMORY;
   plan.grid = (int)grid;
   plan.ctas = ctas;
-  return ensure_workspace(S, workspace_words(ctas, plan.ws_words) * sizeof(uint32_t));
+  const size_t enough = workspace_words(grid, plan.ws_words) * sizeof(uint32_t);
+  int rc = ensure_workspace(S, workspace_words(ctas, plan.ws_words) * sizeof(uint32_t), enough);
+  if (rc == QFS_ERR_NO_MEMORY && ctas > grid) {   // no memory for the crews' CTAs: a CTA for each quartic
+    for (int &crews : plan.crews) crews = 0;
+    plan.ctas = grid;
+    rc = ensure_workspace(S, enough, enough);
+  }
+  return rc;
 }
 
 }  // namespace
@@ -847,7 +862,12 @@ extern "C" int qfs_theta_matrix(int p, int64_t n, const uint8_t *coeffs, uint8_t
   // few quartics: a crew of CTAs for each (p >= 7), as many as the device holds at once
   int crew = 1;
   while (p >= 7 && crew < 8 && 2 * crew * batch <= std::min<int64_t>(2 * (int64_t)S->sms, fit)) crew *= 2;
-  rc = ensure_workspace(*S, workspace_words(batch * crew, stride) * sizeof(uint32_t));
+  const size_t enough = workspace_words(batch, stride) * sizeof(uint32_t);
+  rc = ensure_workspace(*S, workspace_words(batch * crew, stride) * sizeof(uint32_t), enough);
+  if (rc == QFS_ERR_NO_MEMORY && crew > 1) {   // no memory for the crews' CTAs
+    crew = 1;
+    rc = ensure_workspace(*S, enough, enough);
+  }
   if (rc) return rc;
   if (S->which_n < batch) {
     if (S->which) cudaFree(S->which);
@@ -880,20 +900,30 @@ extern "C" int qfs_matmul_mod(int p, int n, int m, int k, const uint8_t *A, cons
   DeviceState *S = nullptr;
   int rc = device_state(&S);
   if (rc) return rc;
-  const size_t need = matmul_scratch_bytes(p, n, m, k);
+  // All rows of A at once; where the scratch does not fit, blocks of rows, each with its own pack of B.
+  int rows = n;
+  size_t need = matmul_scratch_bytes(p, rows, m, k);
   if (S->mm_bytes < need) {
     if (S->mm && cudaFree(S->mm) != cudaSuccess) return cuda_fail(cudaGetLastError());
     S->mm = nullptr;
     S->mm_bytes = 0;
-    if (cudaMalloc(&S->mm, need) != cudaSuccess) {
+    while (cudaMalloc(&S->mm, need) != cudaSuccess) {
+      S->mm = nullptr;
       (void)cudaGetLastError();
-      return QFS_ERR_NO_MEMORY;
+      if (rows <= kMinRowBlock) return QFS_ERR_NO_MEMORY;
+      rows = std::max(kMinRowBlock, (rows + 1) / 2);
+      need = matmul_scratch_bytes(p, rows, m, k);
     }
     S->mm_bytes = need;
   }
-  cudaError_t e = matmul_mod_launch(p, n, m, k, A, B, C, static_cast<uint8_t *>(S->mm), S->sms,
-                                    reinterpret_cast<uint32_t *>(static_cast<char *>(S->ctrl) + 8), stream);
-  return e == cudaSuccess ? QFS_OK : cuda_fail(e);
+  for (int i = 0; i < n; i += rows) {
+    const cudaError_t e = matmul_mod_launch(p, std::min(rows, n - i), m, k, A + (size_t)i * k, B, C + (size_t)i * m,
+                                            static_cast<uint8_t *>(S->mm), S->sms,
+                                            reinterpret_cast<uint32_t *>(static_cast<char *>(S->ctrl) + 8), stream);
+    if (e != cudaSuccess) return cuda_fail(e);
+    if (n - i <= rows) break;
+  }
+  return QFS_OK;
 }
 
 extern "C" int qfs_poly_power(int d, const uint32_t *coeffs, int n, uint32_t *out, cudaStream_t stream) {
@@ -910,19 +940,23 @@ extern "C" int qfs_poly_power(int d, const uint32_t *coeffs, int n, uint32_t *ou
   DeviceState *S = nullptr;
   int rc = device_state(&S);
   if (rc) return rc;
-  const size_t need = polypow_scratch_words(d, n, nprimes) * sizeof(uint32_t);
+  int at_once = polypow_primes_at_once(d, n, nprimes);
+  size_t need = polypow_scratch_words(d, n, nprimes, at_once) * sizeof(uint32_t);
   if (S->pp_bytes < need) {
     if (S->pp && cudaFree(S->pp) != cudaSuccess) return cuda_fail(cudaGetLastError());
     S->pp = nullptr;
     S->pp_bytes = 0;
-    if (cudaMalloc(&S->pp, need) != cudaSuccess) {
+    while (cudaMalloc(&S->pp, need) != cudaSuccess) {
+      S->pp = nullptr;
       (void)cudaGetLastError();
-      return QFS_ERR_NO_MEMORY;
+      if (at_once == 1) return QFS_ERR_NO_MEMORY;
+      at_once = 1;   // one prime after another takes the least
+      need = polypow_scratch_words(d, n, nprimes, at_once) * sizeof(uint32_t);
     }
     S->pp_bytes = need;
   }
   uint32_t *scratch = static_cast<uint32_t *>(S->pp);
-  cudaError_t e = polypow_launch(d, n, nprimes, coeffs, out, scratch, stream);
+  cudaError_t e = polypow_launch(d, n, nprimes, at_once, coeffs, out, scratch, stream);
   return e == cudaSuccess ? QFS_OK : cuda_fail(e);
 }
 

@@ -774,16 +774,19 @@ constexpr size_t kTwWords = 2 * (4096 + 4096 + kPassR / 2);
 // Primes whose transforms run side by side in one launch.  A transform of 2^20 words fills the device for a few
 // microseconds only, so small ones go together (n = 5, two primes: 18 launches and 124 us one after another); 64 MB of
 // them stay in L2 between the passes, which is where the line lies (n = 15: one prime of 64 MB at a time).
-int primes_at_once(uint32_t N, int nprimes) {
+int polypow_primes_at_once(int d, int n, int nprimes) {
+  const int B = d * n + 1;
+  uint32_t N = 1;
+  while ((uint64_t)N < (uint64_t)B * B * B) N <<= 1;
   const uint32_t fit = (64u << 20) / 4u / N;
   return fit < 1 ? 1 : fit < (uint32_t)nprimes ? (int)fit : nprimes;
 }
 
-size_t polypow_scratch_words(int d, int n, int nprimes) {
+size_t polypow_scratch_words(int d, int n, int nprimes, int at_once) {
   const int B = d * n + 1;
   uint32_t N = 1;
   while ((uint64_t)N < (uint64_t)B * B * B) N <<= 1;
-  return (size_t)primes_at_once(N, nprimes) * N + 2 * kTwWords * (size_t)nprimes + (size_t)nprimes * tet(d * n + 1) +
+  return (size_t)at_once * N + 2 * kTwWords * (size_t)nprimes + (size_t)nprimes * tet(d * n + 1) +
          tet(d + 1) + 64;
 }
 
@@ -876,16 +879,15 @@ void column_pass(int kp, uint32_t blocks, uint32_t *a, int logN, int logM, const
 
 }  // namespace
 
-cudaError_t polypow_launch(int d, int n, int nprimes, const uint32_t *coeffs, uint32_t *out, uint32_t *scratch,
-                           cudaStream_t st) {
+cudaError_t polypow_launch(int d, int n, int nprimes, int at_once, const uint32_t *coeffs, uint32_t *out,
+                           uint32_t *scratch, cudaStream_t st) {
   const int B = d * n + 1, D = d * n;
   uint32_t N = 1;
   int logN = 0;
   while ((uint64_t)N < (uint64_t)B * B * B) { N <<= 1; ++logN; }
   const int n_out = tet(D + 1);
   uint32_t *a = scratch;
-  const int group = primes_at_once(N, nprimes);       // transforms side by side
-  uint32_t *tw = a + (size_t)group * N;               // forward and inverse tables of every prime
+  uint32_t *tw = a + (size_t)at_once * N;             // forward and inverse tables of every prime
   uint32_t *res = tw + 2 * kTwWords * (size_t)nprimes;
   const int block = 256;
   // passes: the innermost takes min(8, logN) stages on contiguous runs; the rest, outermost first, up to 8 each
@@ -933,8 +935,8 @@ cudaError_t polypow_launch(int d, int n, int nprimes, const uint32_t *coeffs, ui
     if (e != cudaSuccess) return e;
     coeffs_dev = dev;
   }
-  for (int j = 0; j < nprimes; j += group) {
-    const int count = nprimes - j < group ? nprimes - j : group;
+  for (int j = 0; j < nprimes; j += at_once) {
+    const int count = nprimes - j < at_once ? nprimes - j : at_once;
     const Primes G = Q.from(j);
     const uint32_t runs = (PR.cleared + B - 1) / B;
     fill_kernel<<<dim3(runs / 8 + 1 < 1216 ? runs / 8 + 1 : 1216, count), block, 0, st>>>(given, coeffs_dev, d, B,

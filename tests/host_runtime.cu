@@ -118,14 +118,19 @@ cudaError_t theta_matrix_launch(int, const uint8_t *, int n, int crew, uint8_t *
   return cudaSuccess;
 }
 size_t matmul_scratch_bytes(int, int n, int m, int k) { return (size_t)(n + m) * k; }
-cudaError_t matmul_mod_launch(int, int, int, int, const uint8_t *, const uint8_t *, uint8_t *, uint8_t *, int, uint32_t *,
-                              cudaStream_t) {
+cudaError_t matmul_mod_launch(int, int n, int m, int k, const uint8_t *A, const uint8_t *, uint8_t *C, uint8_t *, int,
+                              uint32_t *, cudaStream_t) {
+  fake::record("matmul n=%d m=%d k=%d a=%zu c=%zu", n, m, k, (size_t)(uintptr_t)A, (size_t)(uintptr_t)C);
   return cudaSuccess;
 }
-int polypow_primes(uint64_t, int) { return 1; }
-size_t polypow_scratch_words(int, int, int) { return 1; }
+int polypow_primes(uint64_t, int) { return 5; }
+int polypow_primes_at_once(int, int, int nprimes) { return nprimes; }
+size_t polypow_scratch_words(int, int, int, int at_once) { return size_t(at_once) << 20; }
 void polypow_plan(int, int, int, uint64_t *, uint64_t *) {}
-cudaError_t polypow_launch(int, int, int, const uint32_t *, uint32_t *, uint32_t *, cudaStream_t) { return cudaSuccess; }
+cudaError_t polypow_launch(int, int, int, int at_once, const uint32_t *, uint32_t *, uint32_t *, cudaStream_t) {
+  fake::record("poly_power at_once=%d", at_once);
+  return cudaSuccess;
+}
 int noalloc_take_counters(uint32_t *, unsigned long long *) { return 0; }
 }  // namespace qfs
 
@@ -170,6 +175,7 @@ int main(int argc, char **argv) {
     fake::live = fake::peak = 0;
     int rc = -1;
     const std::string op = m["op"];
+    if (m.count("after")) qfs_plan_prepare((int)num("after", 7), 1);   // an earlier call's workspace
     if (op == "heights") {   // groups p1, n1, p2, n2, ...
       qfs_group_t g[QFS_MAX_GROUPS];
       int n = 0;
@@ -197,6 +203,12 @@ int main(int argc, char **argv) {
       rc = qfs_plan_prepare((int)num("p", 7), num("n", 0));
     } else if (op == "theta_matrix") {
       rc = qfs_theta_matrix((int)num("p", 7), num("n", 1), rows, rows, nullptr);
+    } else if (op == "matmul") {   // operands at made-up addresses, which nothing reads
+      rc = qfs_matmul_mod(11, (int)num("n", 1), (int)num("m", 1), (int)num("k", 1), reinterpret_cast<uint8_t *>(1 << 20),
+                          rows, reinterpret_cast<uint8_t *>(1 << 20), nullptr);
+    } else if (op == "poly_power") {
+      static uint32_t c[4], limbs[1];
+      rc = qfs_poly_power(1, c, 2, limbs, nullptr);
     }
     std::printf("{\"crews\": [%d, %d, %d, %d], \"crew_for\": [", fake::crews[0], fake::crews[1], fake::crews[2],
                 fake::crews[3]);

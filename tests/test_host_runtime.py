@@ -110,3 +110,47 @@ def test_mixed_launch_on_a_small_budget_uses_its_ctas(runtime):
         r = runtime(op="heights", p1=5, n1=3000, p2=11, n2=30, budget=ctas * 2 * 5052676 * 4)
         assert r["rc"] == 0 and len(r["fused"]) == 1
         assert r["fused"][0]["grid"] >= ctas - ctas // 8
+
+
+CTA_BYTES = {p: 8 * w for p, w in {7: 245904, 11: 5052676, 13: 13138404}.items()}   # two chain buffers
+
+
+@pytest.mark.parametrize("p,n", [(7, 1), (7, 20), (11, 3), (13, 1)])
+def test_no_memory_for_crews_runs_without_them(runtime, p, n):
+    # memory for a CTA per quartic, but not for the CTAs of a crew: the call runs as it did without crews
+    limit = n * CTA_BYTES[p] + 8 * n + CONTROL_BYTES
+    r = runtime(op="heights", p1=p, n1=n, limit=limit)
+    assert r["rc"] == 0 and [f["crew"] for f in r["fused"]] == [1] and r["fused"][0]["grid"] == n
+    assert runtime(op="heights", p1=p, n1=n, limit=CTA_BYTES[p] // 2)["rc"] == 5
+    assert len(runtime(op="heights", p1=p, n1=n)["fused"]) > 1
+    assert runtime(op="prepare", p=p, n=n, limit=limit)["rc"] == 0
+    r = runtime(op="theta_matrix", p=p, n=n, limit=limit)
+    assert r["rc"] == 0 and r["launches"] == [f"theta_matrix n={n} crew=1"]
+    assert runtime(op="theta_matrix", p=p, n=n)["launches"] == [f"theta_matrix n={n} crew=8"]
+    r = runtime(op="heights", p1=p, n1=n, p2=3, n2=2, limit=(n + 2) * CTA_BYTES[p] + 8 * (n + 2) + CONTROL_BYTES)
+    assert r["rc"] == 0 and [f["crew"] for f in r["fused"]] == [1]
+
+
+def test_products_and_powers_without_memory_for_all_at_once(runtime):
+    # (the harness's scratch sizes: (n + m) k bytes, 4 MB per prime side by side)
+    n, m, k = 20001, 7000, 9000
+    r = runtime(op="matmul", n=n, m=m, k=k)
+    assert r["launches"] == [f"matmul n={n} m={m} k={k} a={MB} c={MB}"]
+    r = runtime(op="matmul", n=n, m=m, k=k, limit=13000 * k)
+    done = 0
+    for x in r["launches"]:
+        rows, a, c = (int(re.search(rf"\b{key}=(\d+)", x).group(1)) for key in "nac")
+        assert (a, c) == (MB + done * k, MB + done * m) and (rows + m) * k <= 13000 * k
+        done += rows
+    assert r["rc"] == 0 and done == n
+    assert runtime(op="matmul", n=n, m=m, k=k, limit=m * k)["rc"] == 5
+    assert runtime(op="poly_power")["launches"] == ["poly_power at_once=5"]
+    assert runtime(op="poly_power", limit=19 * MB)["launches"] == ["poly_power at_once=1"]
+    assert runtime(op="poly_power", limit=3 * MB)["rc"] == 5
+
+
+def test_a_workspace_that_suffices_is_kept(runtime):
+    # a call that would like crews, beside a workspace for one quartic: without memory for both it keeps the old one
+    one = runtime(op="prepare", p=11, n=1)["live"]
+    r = runtime(op="theta_matrix", p=7, n=30, after=11, limit=one + 20 * MB)
+    assert r["rc"] == 0 and r["launches"] == ["theta_matrix n=30 crew=1"] and r["live"] <= one + MB
