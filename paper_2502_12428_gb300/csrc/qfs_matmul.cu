@@ -36,9 +36,11 @@ constexpr int kBM = 128, kBN = 256, kBK = 128;   // output tile, and bytes of K 
 constexpr int kTileA = kBM * kBK, kTileB = kBN * kBK;
 constexpr int kMMThreads = 192;                  // warps: TMA, MMA, four that drain
 constexpr int kPackTile = 64;
+constexpr int kRowWords = kBN / 4 + 1;           // a tile's row on its way to an unaligned C: an odd pitch, and a word more to read
 
 __host__ __device__ constexpr int stages_of(int planes) { return 4 / planes; }
-__host__ __device__ constexpr size_t mm_smem(int planes) { return (size_t)stages_of(planes) * planes * (kTileA + kTileB) + 1024; }
+__host__ __device__ constexpr size_t ring_bytes(int planes) { return (size_t)stages_of(planes) * planes * (kTileA + kTileB); }
+__host__ __device__ constexpr size_t mm_smem(int planes) { return ring_bytes(planes) + 1024 + 4 * kBM * kRowWords; }
 
 // ------------------------------------------------------------------------------------------------ pack
 // e4m3 code of an integer with at most four significant bits, |x| <= 128
@@ -306,6 +308,7 @@ __global__ void __launch_bounds__(kMMThreads, 1)
     bool ok = true;
     for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
       const int i = (tile % tiles_n) * kBM + 32 * quad + lane, j0 = (tile / tiles_n) * kBN;
+      const int len = min(kBN, m - j0);
       uint32_t res[kBN / 4];   // residues of the chunks so far, four to a word
 #pragma unroll
       for (int w = 0; w < kBN / 4; ++w) res[w] = 0;
@@ -316,6 +319,7 @@ __global__ void __launch_bounds__(kMMThreads, 1)
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
         for (int c = 0; c < kBN; c += 32) {
+          if (c >= len) continue;   // columns past the end of C
           uint32_t v[32];
           tmem_ld32(tmem + ((uint32_t)(32 * quad) << 16) + a * kBN + c, v);
 #pragma unroll
@@ -332,34 +336,57 @@ __global__ void __launch_bounds__(kMMThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(&tempty[a]);
       }
-      if (ok && i < n) {
-        uint8_t *row = C + (size_t)i * m + j0;
-        const int len = min(kBN, m - j0);
+      if (!ok) break;
+      if (vec >= 4) {
+        if (i < n) {
+          uint8_t *row = C + (size_t)i * m + j0;
 #pragma unroll
-        for (int w = 0; w < kBN / 4; w += 4) {
-          if (vec >= 16 && 4 * w + 16 <= len) {
-            *reinterpret_cast<uint4 *>(row + 4 * w) = make_uint4(res[w], res[w + 1], res[w + 2], res[w + 3]);
-            continue;
-          }
-#pragma unroll
-          for (int x = w; x < w + 4; x += 2) {
-            if (vec >= 8 && 4 * x + 8 <= len) {
-              *reinterpret_cast<uint2 *>(row + 4 * x) = make_uint2(res[x], res[x + 1]);
+          for (int w = 0; w < kBN / 4; w += 4) {
+            if (vec >= 16 && 4 * w + 16 <= len) {
+              *reinterpret_cast<uint4 *>(row + 4 * w) = make_uint4(res[w], res[w + 1], res[w + 2], res[w + 3]);
               continue;
             }
 #pragma unroll
-            for (int y = x; y < x + 2; ++y) {
-              if (vec >= 4 && 4 * y + 4 <= len) {
-                *reinterpret_cast<uint32_t *>(row + 4 * y) = res[y];
-              } else {
-#pragma unroll
-                for (int b = 0; b < 4; ++b)
-                  if (4 * y + b < len) row[4 * y + b] = (uint8_t)(res[y] >> (8 * b));
+            for (int x = w; x < w + 4; x += 2) {
+              if (vec >= 8 && 4 * x + 8 <= len) {
+                *reinterpret_cast<uint2 *>(row + 4 * x) = make_uint2(res[x], res[x + 1]);
+                continue;
               }
+#pragma unroll
+              for (int y = x; y < x + 2; ++y)
+                if (4 * y < len) *reinterpret_cast<uint32_t *>(row + 4 * y) = res[y];   // (len: a multiple of four)
             }
           }
         }
+        continue;
       }
+      // Rows of C at odd addresses: the warp's 32 rows go through shared memory and out as aligned words, a row (several
+      // rows, where they are short) at a time, instead of as single bytes of 32 rows at a time.  mod 31, n = m = 4,097,
+      // k = 129: 169 us by bytes, 43 so (rows of 4,096: 29).
+      uint32_t *rows = reinterpret_cast<uint32_t *>(smem_raw + (stage0 - smem_u32(smem_raw)) + ring_bytes(PLANES)) +
+                       32 * quad * kRowWords;
+#pragma unroll
+      for (int w = 0; w < kBN / 4; ++w)
+        if (4 * w < len) rows[lane * kRowWords + w] = res[w];
+      __syncwarp();
+      int per_row = 32;   // lanes of a row
+      while (per_row > 1 && 4 * (per_row / 2) >= len + 3) per_row /= 2;
+      const int sub = lane & (per_row - 1), step = 32 / per_row, n_rows = min(32, n - (i - lane));
+#pragma unroll 4
+      for (int r = lane / per_row; r < n_rows; r += step) {
+        const uint32_t *src = rows + r * kRowWords;
+        const uint8_t *bytes = reinterpret_cast<const uint8_t *>(src);
+        uint8_t *dst = C + (size_t)(i - lane + r) * m + j0;
+        const int head = min(len, (int)(-reinterpret_cast<uintptr_t>(dst) & 3)), words = (len - head) >> 2;
+        const int edges = len - 4 * words;   // bytes before the first aligned word and after the last
+        for (int w = sub; w < words; w += per_row)   // bytes head + 4w .. head + 4w + 3
+          *reinterpret_cast<uint32_t *>(dst + head + 4 * w) = __funnelshift_r(src[w], src[w + 1], 8 * head);
+        for (int e = sub; e < edges; e += per_row) {
+          const int at = e < head ? e : e + 4 * words;
+          dst[at] = bytes[at];
+        }
+      }
+      __syncwarp();   // the next tile overwrites the rows
     }
   }
   __syncwarp();

@@ -704,6 +704,36 @@ def test_matmul_mod_unaligned_views(qfs):
         assert not bufs[2][:off].any() and not bufs[2][off + n * m:].any()
 
 
+@pytest.mark.parametrize("p", [11, 251])
+@pytest.mark.parametrize("n,m", [(1, 1), (31, 3), (33, 255), (127, 257), (129, 258), (161, 511), (200, 515)])
+def test_matmul_mod_rows_at_odd_addresses(qfs, p, n, m):
+    # rows of C that start anywhere: first and last words of a row are shared with its neighbours, and nothing else is touched
+    rng = np.random.default_rng(100 * n + m)
+    k = 70
+    A, B = rng.integers(0, p, (n, k), dtype=np.uint8), rng.integers(0, p, (k, m), dtype=np.uint8)
+    want = (A.astype(np.int64) @ B.astype(np.int64) % p).astype(np.uint8)
+    a, b = dev_tensor(A), dev_tensor(B)
+    for off in range(4):
+        buf = torch.full((n * m + 16,), 255, dtype=torch.uint8, device="cuda:0")
+        c = buf[off + 4:off + 4 + n * m].view(n, m)
+        qfs.matmul_mod(p, a, b, out=c)
+        assert np.array_equal(c.cpu().numpy(), want), off
+        assert (buf[:off + 4] == 255).all() and (buf[off + 4 + n * m:] == 255).all()
+    assert qfs.read_status() == 0
+
+
+def test_matmul_mod_odd_row_length_costs_little(qfs):
+    # a short product with odd rows is bound by its stores, as is one with aligned rows
+    def ms(n):
+        g = torch.Generator(device="cuda").manual_seed(n)
+        A = torch.randint(0, 31, (n, 129), dtype=torch.uint8, device="cuda", generator=g)
+        B = torch.randint(0, 31, (129, n), dtype=torch.uint8, device="cuda", generator=g)
+        out = torch.empty(n, n, dtype=torch.uint8, device="cuda")
+        return _ms(lambda: [qfs.matmul_mod(31, A, B, out=out) for _ in range(10)])
+    even, odd = ms(4096), ms(4097)
+    assert odd < 2 * even, (odd, even)
+
+
 def test_matmul_mod_long_k_reduces_between_tiles(qfs):
     # k (p-1)^2 above 2^31 at p = 251: the accumulators are reduced between K tiles
     p, n, m, k = 251, 16, 24, 40000
