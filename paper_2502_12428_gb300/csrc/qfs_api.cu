@@ -451,8 +451,7 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
     // shared memory: the largest iterate pair of the launch plus the largest ring any group's tile needs
     int ring_words = 0;
     for (int i = 0; i < prm.n_groups; ++i)
-      ring_words = std::max(ring_words, ring_words_for(prm.g[i].p, tile_for(prm.g[i].p),
-                                                       uses_ring_chain(form, prm.g[i].p), power));
+      ring_words = std::max(ring_words, ring_words_of(form, prm.g[i].p, tile_for(prm.g[i].p), power));
     const size_t smem = ring_offset_for(tet(4 * (max_p - 1) + 1)) + 4 * (size_t)ring_words;
     rc = make_plan(*S, form, max_p, n_items, opts, plan, smem,
                    form == QFS_FORM_DP4A && power == QFS_POWER_CHAIN ? &prm : nullptr);
@@ -517,7 +516,7 @@ int qfs_plan_prepare(int p, int64_t n_hint) {
   Plan plan;
   int64_t n = n_hint > 0 ? n_hint : (int64_t)1 << 40;
   for (int form : {QFS_FORM_INT32, QFS_FORM_DP4A, QFS_FORM_INT8TC}) {
-    rc = make_plan(*S, form, p, n, nullptr, plan, smem_bytes_for(p, tile_for(p), uses_ring_chain(form, p)));
+    rc = make_plan(*S, form, p, n, nullptr, plan, smem_bytes_of(form, p, tile_for(p)));
     if (rc) return rc;
   }
   {   // the dp4a chain's own launches, crews included
@@ -526,8 +525,7 @@ int qfs_plan_prepare(int p, int64_t n_hint) {
     prm.n_groups = 1;
     prm.g[0].p = p;
     prm.g[0].n = n;
-    const size_t smem = ring_offset_for(tet(4 * (p - 1) + 1)) +
-                        4 * (size_t)ring_words_for(p, tile_for(p), uses_ring_chain(QFS_FORM_DP4A, p), QFS_POWER_CHAIN);
+    const size_t smem = smem_bytes_of(QFS_FORM_DP4A, p, tile_for(p), QFS_POWER_CHAIN);
     rc = make_plan(*S, QFS_FORM_DP4A, p, n, nullptr, plan, smem, &prm);
     if (rc) return rc;
   }
@@ -678,8 +676,7 @@ int qfs_sweep_autotune(int form, int p, int64_t n, const uint8_t *coeffs, int *b
   slot = SweepConfig{0, 0};
   int max_ctas = 1;
   {
-    const size_t smem = ring_offset_for(tet(4 * (p - 1) + 1)) +
-                        4 * (size_t)ring_words_for(p, tile_for(p), uses_ring_chain(form, p), QFS_POWER_CHAIN);
+    const size_t smem = smem_bytes_of(form, p, tile_for(p), QFS_POWER_CHAIN);
     int blocks = 0;
     if (form_occupancy(form, &blocks, smem, false) == cudaSuccess) max_ctas = std::max(1, blocks);
   }

@@ -98,34 +98,35 @@ __host__ __device__ inline int chain_slot_words(int p, TileConfig tc) {
 
 __host__ __device__ inline int theta_ring_words_for(int p, int power = -1);
 
-// Ring words the identity and reduced power modes need: three byte arrays (f^(p-2), Delta_1(f), E), and in the
-// reduced mode a product to degree 4p whose own ring starts after f^(p-2), Delta_1(f) and q.
-__host__ __device__ inline int aux_ring_words(int p, TileConfig tc, bool ring_chain) {
+// Ring words of the byte arrays of one power mode (-1: every mode): f^(p-2), Delta_1(f) and E in the identity mode, f^(p-2),
+// Delta_1(f) and the 35 taps q in the reduced mode.  The modes' chain products run before the arrays lie there.
+__host__ __device__ inline int aux_ring_words(int p, int power) {
   const int l_fpm2 = tet(4 * (p - 2) + 1), l_d1f = tet(4 * p + 1), l_E = tet(4 * (p - 1) + 1);
-  const int ring_off = (((l_fpm2 + l_d1f + 3) / 4 + 64) + 3) & ~3;
-  int chain = block_ring_words(p);
-  if (ring_chain)
-    for (int s0 = 0; s0 <= 4 * p; s0 += 32) {
-      const ChainTile T = chain_tile(s0, 4 * p, tc);
-      chain = max(chain, T.nslot * T.slot_words);
-    }
-  return max(ring_off + chain, (l_fpm2 + l_d1f + l_E + 3) / 4);
+  return max(power == 0 || power == 1 ? 0 : (l_fpm2 + l_d1f + 3) / 4 + 1 + 35,
+             power == 0 || power == 2 ? 0 : (l_fpm2 + l_d1f + l_E + 3) / 4);
 }
 
 // Which chain product a form runs at prime p: the shared-memory slice ring (the int8 tensor form, whose tiles read
-// aligned words of a staged slice), or one that needs no more than block_ring_words (dp4a and int32 forms).
+// aligned words of a staged slice), strips staged by blocks (dp4a form, qfs_block.cuh), or lane sweeps, which stage
+// nothing (int32 form).
 __host__ __device__ constexpr bool uses_ring_chain(int form, int p) { return form == 2 && p > 0; }
+__host__ __device__ constexpr bool uses_blocks(int form) { return form == 1; }
 
-// Shared-memory ring words for prime p: the chain's slice ring (the int8 tensor form's, or the dp4a form's strips),
-// theta's Delta slots, and the power modes' arrays.  ring_chain = true gives the size every form fits in;
-// power (QFS_POWER_*, -1 for every mode) sizes theta for one power mode.
-__host__ __device__ inline int ring_words_for(int p, TileConfig tc, bool ring_chain = true, int power = -1) {
-  return max(max(max(ring_chain ? chain_slot_words(p, tc) : 0, block_ring_words(p)), theta_ring_words_for(p, power)),
-             power != 0 ? aux_ring_words(p, tc, ring_chain) : 0);
+// Shared-memory ring words of a launch of one form at prime p: what its chain product stages, theta's Delta slots, and
+// the power modes' arrays.  power (QFS_POWER_*, -1 for every mode) sizes theta and the arrays for one power mode.  At p = 13
+// the dp4a product's strips leave room for two CTAs per SM and for nothing else.
+__host__ __device__ inline int ring_words_of(int form, int p, TileConfig tc, int power = -1) {
+  return max(max(uses_ring_chain(form, p) ? chain_slot_words(p, tc) : uses_blocks(form) ? block_ring_words(p) : 0,
+                 theta_ring_words_for(p, power)),
+             aux_ring_words(p, power));
 }
-
+__host__ __device__ inline size_t smem_bytes_of(int form, int p, TileConfig tc, int power = -1) {
+  return ring_offset_for(tet(4 * (p - 1) + 1)) + 4 * (size_t)ring_words_of(form, p, tc, power);
+}
+// The size that every form fits in (ring_chain), or the dp4a and int32 forms.
 __host__ __device__ inline size_t smem_bytes_for(int p, TileConfig tc, bool ring_chain = true) {
-  return ring_offset_for(tet(4 * (p - 1) + 1)) + 4 * (size_t)ring_words_for(p, tc, ring_chain);
+  const size_t blocks = smem_bytes_of(1, p, tc), ring = smem_bytes_of(2, p, tc);
+  return ring_chain && ring > blocks ? ring : blocks;
 }
 __host__ __device__ inline size_t smem_bytes_for(int p, bool ring_chain = true) {
   return smem_bytes_for(p, default_tile(p), ring_chain);
@@ -1498,22 +1499,20 @@ __device__ __noinline__ int reduced_height(Smem &sm, uint8_t *gs, uint8_t *gn, u
   uint8_t *fpm2 = reinterpret_cast<uint8_t *>(ring);
   uint8_t *d1f = fpm2 + l_fpm2;
   int *q = reinterpret_cast<int *>(ring + (l_fpm2 + l_d1f + 3) / 4 + 1);
-  // f^(p-2) mod p from `other` (degree dm)
+  // f^(p-2) mod p from `other` (degree dm), in the second iterate's place while the product below stages in the ring
   for (int k = tid; k < sm.SW[dm + 1] / 4; k += nthreads) {
     int u, s, c;
     decode_form_chunk(k, dm, sm.SW, u, s, c);
     const uint4 v = *reinterpret_cast<const uint4 *>(other + 4 * k);
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
     for (int b = 0; b < 16 && 16 * c + b <= s; ++b)
-      fpm2[tet(u) + tri(s) + 16 * c + b] = (uint8_t)(((w[b >> 2] >> (8 * (b & 3))) & 0xFFu) % P);
+      gn[tet(u) + tri(s) + 16 * c + b] = (uint8_t)(((w[b >> 2] >> (8 * (b & 3))) & 0xFFu) % P);
   }
   __syncthreads();
   // f~^p = f~^(p-1) f~ (mod p^2), then Delta_1(f) = (f~^p - sum a~_I^p x^(pI)) / p mod p
-  // the product's slot ring goes after fpm2, d1f and q, on a 16-byte boundary (16-byte cp.async and loads)
-  constexpr int ring_off = (((l_fpm2 + l_d1f + 3) / 4 + 64) + 3) & ~3;   // same offset as aux_ring_words
-  static_assert(ring_off % 4 == 0, "16-byte aligned ring");
-  chain_step_call<P, FORM, DEBUG>(cur, other, d, sm, ring + ring_off, gs, status, dbg);
+  chain_step_call<P, FORM, DEBUG>(cur, other, d, sm, ring, gs, status, dbg);
   __syncthreads();
+  for (int i = tid; i < l_fpm2; i += nthreads) fpm2[i] = gn[i];
   bool bad = false;
   for (int k = tid; k < sm.SW[d1 + 1] / 4; k += nthreads) {
     int u, s, c;

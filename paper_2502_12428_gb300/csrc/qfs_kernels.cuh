@@ -118,7 +118,7 @@ struct FormLauncher {
   cudaError_t FormLauncher<FORM>::debug(int p, const uint8_t *f, int max_h, int8_t *h_out, uint32_t *bufA,    \
                                         uint32_t *bufB, uint32_t *status, DebugPtrs dbg, cudaStream_t st,     \
                                         int power_mode) {                                                     \
-    const size_t smem = smem_bytes_for(p, uses_ring_chain(FORM, p));                                         \
+    const size_t smem = smem_bytes_of(FORM, p, default_tile(p));                                              \
     cudaError_t e = cudaSuccess;                                                                              \
     switch (p) {                                                                                              \
       case 3: QFS_DEBUG_LAUNCH(3, FORM); break;                                                               \

@@ -116,7 +116,7 @@ extern "C" int qfs_heights_noalloc(int p, int64_t n, const uint8_t *coeffs, int 
   int rc = scratch_for_current_device(&scratch, &sms, &fresh);
   if (rc) return rc;
 
-  const size_t smem = smem_bytes_for(p, uses_ring_chain(QFS_FORM_DP4A, p));
+  const size_t smem = smem_bytes_of(QFS_FORM_DP4A, p, default_tile(p), QFS_POWER_CHAIN);
   cudaError_t e = cudaFuncSetAttribute(noalloc_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return QFS_ERR_CUDA;

@@ -102,7 +102,7 @@ template <int P>
 cudaError_t launch(const uint8_t *coeffs, int n, int crew, uint8_t *M, uint32_t *ws, size_t stride, int *which,
                    uint32_t *status, cudaStream_t st) {
   using Pr = Prime<P>;
-  const size_t smem = smem_bytes_for(P, uses_ring_chain(QFS_FORM_DP4A, P));
+  const size_t smem = smem_bytes_of(QFS_FORM_DP4A, P, default_tile(P), QFS_POWER_CHAIN);
   cudaError_t e = cudaFuncSetAttribute(theta_delta_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   e = launch_crews(theta_delta_kernel<P>, n * crew, crew, smem, st, coeffs, ws, stride, which, status);

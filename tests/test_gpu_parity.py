@@ -626,6 +626,21 @@ def test_reduced_kernel_and_general_route(qfs, p, n):
         assert np.array_equal(got[1].cpu().numpy(), oracle.heights(q, g))
 
 
+@pytest.mark.parametrize("p,n", [(3, 300), (5, 300), (7, 200), (11, 150), (13, 150)])
+@pytest.mark.parametrize("form", CORE_FORMS)
+def test_reduced_mode_in_the_fused_kernel(qfs, p, n, form):
+    # f^(p-2) waits in the second iterate's place while the product to f~^p stages in the ring
+    f = np.concatenate([inputs.dense(p, n, 9980 + p), inputs.sparse(p, n, 9990 + p)])
+    want = oracle.heights(p, f)
+    assert len(set(want.tolist())) >= 3
+    t = dev_tensor(f)
+    assert np.array_equal(qfs.heights(p, t, power="reduced", form=form, max_ctas=200).cpu().numpy(), want)
+    row = f[np.flatnonzero(want > 2)[0]]
+    got = qfs.debug_stages(p, dev_tensor(row), form=form, power="reduced")
+    assert got["h"] == want[np.flatnonzero(want > 2)[0]]
+    assert qfs.read_status() == 0
+
+
 def test_reduced_mode_paper_examples(qfs):
     for p in (5, 7, 11, 13):
         sel = [r for r in example_quartics() if r[0] == p]

@@ -154,3 +154,15 @@ def test_a_workspace_that_suffices_is_kept(runtime):
     one = runtime(op="prepare", p=11, n=1)["live"]
     r = runtime(op="theta_matrix", p=7, n=30, after=11, limit=one + 20 * MB)
     assert r["rc"] == 0 and r["launches"] == ["theta_matrix n=30 crew=1"] and r["live"] <= one + MB
+
+
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("power", [0, 1, 2])
+@pytest.mark.parametrize("p", [3, 5, 7, 11, 13])
+def test_two_ctas_per_sm_in_every_mode(runtime, p, power, form):
+    # the shared memory of a launch: two CTAs share an SM at every prime, and a form pays only for its own product
+    r = runtime(op="heights", p1=p, n1=100000, power=power, form=form, max_ctas=10 ** 6)
+    assert [f["grid"] for f in r["fused"]] == [2 * 152]
+    if form == 0 and power == 2:   # nothing is staged: the iterates and the mode's byte arrays
+        ld, fpm2, d1f = ((d + 1) * (d + 2) * (d + 3) // 6 for d in (4 * (p - 1), 4 * (p - 2), 4 * p))
+        assert r["fused"][0]["smem"] <= 6000 + 2 * ld + fpm2 + d1f + 300
