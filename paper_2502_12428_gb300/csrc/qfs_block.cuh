@@ -50,26 +50,36 @@ namespace block {
 constexpr int kSlices = 4;   // output slices of a block, input slices of a group
 constexpr int kGroups = 3;   // staged groups of a team: two being read, one in flight
 // Threads of a team: the strips of a small team are short, which leaves fewer threads waiting for the strip's later
-// columns; at p >= 11 the rings of several teams would not fit in shared memory.
-__host__ __device__ constexpr int team_threads(int p) { return p <= 7 ? 64 : kThreads; }
+// columns; at p >= 11 the rings of several teams would not fit in shared memory.  The products up to f~^p (SMALL, degree
+// 4p at most) fit four teams at every prime, and one team of 256 has a single strip of them to do: f^(p-1) takes
+// 133 us by four teams at p = 11 and 233 by one.
+constexpr int kSmallTeam = 64;
+__host__ __device__ constexpr int team_threads(int p) { return p <= 7 ? kSmallTeam : kThreads; }
+// whether a prime's small products run by other teams than its long ones
+__host__ __device__ constexpr bool small_apart(int p) { return team_threads(p) != kSmallTeam; }
 
 // First item of every strip of the longest product, and of the strip after it: column | half-chunk << 16.
 __device__ __forceinline__ void build_strip_tab(int p, Smem &sm) {
   static_assert(half_prefix(kMaxD + 1) / team_threads(kMaxP) + 2 <= kMaxStrips, "strips of the largest prime");
-  const int team = team_threads(p), n = half_prefix(4 * p * (p - 1) + 1) / team + 2;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    int s, h;
-    decode_half(k * team, s, h);
-    sm.strip_tab[k] = (uint32_t)s | ((uint32_t)h << 16);
-  }
+  static_assert(half_prefix(4 * kMaxP + 1) / kSmallTeam + 2 <= kMaxSmallStrips, "strips of its small products");
+  auto build = [](uint32_t *tab, int team, int degree) {
+    const int n = half_prefix(degree + 1) / team + 2;
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+      int s, h;
+      decode_half(k * team, s, h);
+      tab[k] = (uint32_t)s | ((uint32_t)h << 16);
+    }
+  };
+  build(sm.strip_tab, team_threads(p), 4 * p * (p - 1));
+  if (small_apart(p)) build(sm.small_tab, kSmallTeam, 4 * p);
 }
 
 // Columns s_lo .. s_hi of strip k of a product of degree m_out, staged from column c_lo; h_lo: its first half-chunk.
 struct Strip {
   int s_lo, h_lo, s_hi, c_lo;
 };
-__device__ __forceinline__ Strip strip_at(const Smem &sm, int k, int m_out) {
-  const uint32_t a = sm.strip_tab[k], b = sm.strip_tab[k + 1];
+__device__ __forceinline__ Strip strip_at(const uint32_t *tab, int k, int m_out) {
+  const uint32_t a = tab[k], b = tab[k + 1];
   Strip S;
   S.s_lo = (int)(a & 0xFFFFu);
   S.h_lo = (int)(a >> 16);
@@ -78,11 +88,10 @@ __device__ __forceinline__ Strip strip_at(const Smem &sm, int k, int m_out) {
   return S;
 }
 
-// Words of one staged slice (a zero chunk, then the strip's columns) that every strip of every product of prime p
+// Words of one staged slice (a zero chunk, then the strip's columns) that every strip of every product up to degree D
 // fits in: strips start at multiples of a team's items and a longer product only adds columns at the end, so the
 // strips of the longest form cover all.
-__host__ __device__ constexpr int slice_stride(int p) {
-  const int D = 4 * p * (p - 1), team = team_threads(p);
+__host__ __device__ constexpr int slice_stride(int D, int team) {
   int best = 0, s_lo = 0, first = 0;   // first: items before column s_lo
   for (int i0 = 0; i0 < half_prefix(D + 1); i0 += team) {
     while (first + half_chunks_of(s_lo) <= i0) first += half_chunks_of(s_lo++);
@@ -93,9 +102,10 @@ __host__ __device__ constexpr int slice_stride(int p) {
   }
   return best;
 }
-template <int P>
+template <int P, bool SMALL>
 struct Ring {
-  static constexpr int stride = slice_stride(P);             // words between the slices of a group
+  static constexpr int team = SMALL ? kSmallTeam : team_threads(P);
+  static constexpr int stride = slice_stride(SMALL ? 4 * P : 4 * P * (P - 1), team);   // words between the slices of a group
   static constexpr int group = kSlices * stride;             // words of a group
   static constexpr int words = kGroups * group;              // words of a team's ring
 };
@@ -133,11 +143,11 @@ __device__ __forceinline__ void windows(const Col &x, int q, uint32_t *out) {
 }
 
 // The columns of input slice v = u0 - 4 + K that a block needs: sI <= the largest uI it takes part in.
-template <int P, int K>
+template <int STRIDE, int K>
 __device__ __forceinline__ void load_slice(const char *group, const Lane &L, Col (&x)[5]) {
   constexpr int u_hi = K < 3 ? 4 : 7 - K;
 #pragma unroll
-  for (int c = 0; c <= u_hi; ++c) x[c] = load_col(group + L.off[c] + (K & 3) * 4 * Ring<P>::stride);
+  for (int c = 0; c <= u_hi; ++c) x[c] = load_col(group + L.off[c] + (K & 3) * 4 * STRIDE);
 }
 
 // Input slice v = u0 - 4 + K of a block into the sums of the output slices it feeds (j with uI = j + 4 - K in 0..4).
@@ -241,28 +251,28 @@ __device__ __forceinline__ void store_slice(uint32_t *__restrict__ out, const Sm
 // The block u0 .. u0+3 over every tap pair: groups ga (slices u0-4 .. u0-1) and gb (u0 .. u0+3; absent in the block
 // of the last four output slices, whose inputs end at u0 - 1).  The columns of a slice are loaded while the slice
 // before is multiplied.
-template <int P>
+template <int STRIDE>
 __device__ __forceinline__ void dense_block(const char *ga, const char *gb, bool last, const Lane &L, const Taps &T,
                                             uint32_t (&acc)[kSlices][8]) {
   Col xa[5], xb[5];
-  load_slice<P, 0>(ga, L, xa);
-  load_slice<P, 1>(ga, L, xb);
+  load_slice<STRIDE, 0>(ga, L, xa);
+  load_slice<STRIDE, 1>(ga, L, xb);
   slice_macs<0>(xa, T, acc);
-  load_slice<P, 2>(ga, L, xa);
+  load_slice<STRIDE, 2>(ga, L, xa);
   slice_macs<1>(xb, T, acc);
-  load_slice<P, 3>(ga, L, xb);
+  load_slice<STRIDE, 3>(ga, L, xb);
   slice_macs<2>(xa, T, acc);
   if (last) {
     slice_macs<3>(xb, T, acc);
     return;
   }
-  load_slice<P, 4>(gb, L, xa);
+  load_slice<STRIDE, 4>(gb, L, xa);
   slice_macs<3>(xb, T, acc);
-  load_slice<P, 5>(gb, L, xb);
+  load_slice<STRIDE, 5>(gb, L, xb);
   slice_macs<4>(xa, T, acc);
-  load_slice<P, 6>(gb, L, xa);
+  load_slice<STRIDE, 6>(gb, L, xa);
   slice_macs<5>(xb, T, acc);
-  load_slice<P, 7>(gb, L, xb);
+  load_slice<STRIDE, 7>(gb, L, xb);
   slice_macs<6>(xa, T, acc);
   slice_macs<7>(xb, T, acc);
 }
@@ -287,24 +297,25 @@ __device__ __forceinline__ Unit unit_at(const Strip &S, int j, int seg, int m_ou
 // 1.300) and 12.5 at p = 7 (32 / 16 / 4: level, 8 / 4 / 2: 13.0).
 __device__ __forceinline__ int unit_log2(int m_out) { return m_out >= 120 ? 4 : m_out >= 72 ? 3 : 2; }
 
-template <int P>
+template <int n>
 __device__ __forceinline__ void team_sync(int team) {
-  constexpr int n = team_threads(P);
   if constexpr (n == kThreads) __syncthreads();
   else asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(n) : "memory");
 }
 
-template <int P, bool LAST, bool DEBUG>
+template <int P, bool SMALL, bool LAST, bool DEBUG>
 __device__ __noinline__ void run_strips(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, int m_in,
                                         Smem &sm, uint32_t *ring, const uint8_t *gs, uint32_t *status,
                                         DebugPtrs dbg) {
-  constexpr int kTeam = team_threads(P), kOwn = kThreads / kTeam, kPerSlice = kTeam / kSlices;
-  constexpr int kCopies = (Ring<P>::stride / 4 - 1 + kPerSlice - 1) / kPerSlice;   // 16-byte copies per thread and group
+  using R = Ring<P, SMALL>;
+  constexpr int kTeam = R::team, kOwn = kThreads / kTeam, kPerSlice = kTeam / kSlices;
+  constexpr int kCopies = (R::stride / 4 - 1 + kPerSlice - 1) / kPerSlice;   // 16-byte copies per thread and group
+  const uint32_t *tab = SMALL && small_apart(P) ? sm.small_tab : sm.strip_tab;
   const int m_out = m_in + 4;
   const int n_items = half_prefix(m_out + 1), n_strips = (n_items + kTeam - 1) / kTeam;
   const int team = (int)threadIdx.x / kTeam, tt = (int)threadIdx.x % kTeam;
   const int fs = tt / kPerSlice, fk = tt % kPerSlice;   // slice of a group and first chunk this thread copies
-  ring += team * Ring<P>::words;
+  ring += team * R::words;
   // teams of the crew; a crew's units are shorter, so that there are enough of them
   const int kTeams = kOwn * sm.crew, me = kOwn * sm.rank + team;
   const int lg = max(1, unit_log2(m_out) - (sm.crew > 1 ? high_bit((unsigned)sm.crew) : 0)), seg = 1 << lg;   // blocks of a unit
@@ -319,7 +330,7 @@ __device__ __noinline__ void run_strips(const uint32_t *__restrict__ in, uint32_
 #pragma unroll
   for (int r = 0; r < 4; ++r) T.a00[r] = (uint32_t)sm.taps[0] << (8 * r);
   // the zero chunk before each staged slice
-  if (tt < kGroups * kSlices) *reinterpret_cast<uint4 *>(ring + tt * Ring<P>::stride) = make_uint4(0u, 0u, 0u, 0u);
+  if (tt < kGroups * kSlices) *reinterpret_cast<uint4 *>(ring + tt * R::stride) = make_uint4(0u, 0u, 0u, 0u);
 
   // Unit queue of the product (counter (m_in / 4) mod 2 of the crew's first CTA; the other one is cleared for the next
   // product).  Units are numbered strip after strip; a team's first two are fixed, the others come from the counter.
@@ -337,7 +348,7 @@ __device__ __noinline__ void run_strips(const uint32_t *__restrict__ in, uint32_
   int cur_k = 0, cur_base = 0;   // cursor: strip and the number of units before it
   auto find = [&](int u) {       // unit u >= the last one -> strip | segment << 16, or -1 past the end
     while (cur_k < n_strips) {
-      const int nb = (m_out - (int)(sm.strip_tab[cur_k] & 0xFFFFu) + 4) >> 2;
+      const int nb = (m_out - (int)(tab[cur_k] & 0xFFFFu) + 4) >> 2;
       const int n = (nb + seg - 1) >> lg;
       if (u < cur_base + n) return cur_k | ((u - cur_base) << 16);
       cur_base += n;
@@ -349,7 +360,7 @@ __device__ __noinline__ void run_strips(const uint32_t *__restrict__ in, uint32_
   int fid = find(me), f_g = 0, f_ng = 0, f_v = 0, f_hi = 0, f_base = 0, f_n = 0;
   auto stage_unit = [&]() {
     if (fid < 0) { f_ng = 0; return; }
-    const Strip S = strip_at(sm, fid & 0xFFFF, m_out);
+    const Strip S = strip_at(tab, fid & 0xFFFF, m_out);
     const Unit U = unit_at(S, fid >> 16, seg, m_out);
     f_g = 0;
     f_ng = U.ng;
@@ -379,7 +390,7 @@ __device__ __noinline__ void run_strips(const uint32_t *__restrict__ in, uint32_
     }
     if (f_ng > 0) {
       const int v = f_v + fs;
-      uint32_t *dst = ring + slot * Ring<P>::group + fs * Ring<P>::stride + 4 + 4 * fk;
+      uint32_t *dst = ring + slot * R::group + fs * R::stride + 4 + 4 * fk;
       const uint32_t *src = in + sm.SW[max(v, 0)] + f_base + 4 * fk;
       int have = f_n;
       if (f_v < f_hi) {   // a slice of this group lacks some of the strip's columns: zeros there
@@ -400,7 +411,7 @@ __device__ __noinline__ void run_strips(const uint32_t *__restrict__ in, uint32_
   fetch(0);
   fetch(1);
   while (uid >= 0) {
-    const Strip S = strip_at(sm, uid & 0xFFFF, m_out);
+    const Strip S = strip_at(tab, uid & 0xFFFF, m_out);
     const Unit U = unit_at(S, uid >> 16, seg, m_out);
     const bool top = (uid >> 16) == 0;
     Lane L;
@@ -426,18 +437,18 @@ __device__ __noinline__ void run_strips(const uint32_t *__restrict__ in, uint32_
     for (int b = 0; b < U.ng; ++b, u0 += 4) {
       // this block's groups have arrived for every thread, and nobody reads the slot of the block before any more
       cp_async_wait_all();
-      team_sync<P>(team);
+      team_sync<kTeam>(team);
       const int slot_b = slot == kGroups - 1 ? 0 : slot + 1, slot_f = slot_b == kGroups - 1 ? 0 : slot_b + 1;
       fetch(slot_f);
       if (b < U.nb && u0 + 3 >= s_first) {
-        const char *ga = reinterpret_cast<const char *>(ring + slot * Ring<P>::group);
-        const char *gb = reinterpret_cast<const char *>(ring + slot_b * Ring<P>::group);
+        const char *ga = reinterpret_cast<const char *>(ring + slot * R::group);
+        const char *gb = reinterpret_cast<const char *>(ring + slot_b * R::group);
         uint32_t acc[kSlices][8];
 #pragma unroll
         for (int j = 0; j < kSlices; ++j)
 #pragma unroll
           for (int e = 0; e < 8; ++e) acc[j][e] = 0;
-        dense_block<P>(ga, gb, top && b == U.nb - 1, L, T, acc);
+        dense_block<R::stride>(ga, gb, top && b == U.nb - 1, L, T, acc);
 #pragma unroll
         for (int j = 0; j < kSlices; ++j)
           store_slice<P, LAST, DEBUG>(out, sm, L, u0 + j, gs, acc[j], bad, dbg);
@@ -455,17 +466,21 @@ __device__ __noinline__ void run_strips(const uint32_t *__restrict__ in, uint32_
 
 // Words of shared memory a dp4a product of prime p stages its input in.
 __host__ __device__ constexpr int block_ring_words(int p) {
-  return kThreads / block::team_threads(p) * block::kGroups * block::kSlices * block::slice_stride(p);
+  return kThreads / block::team_threads(p) * block::kGroups * block::kSlices *
+         block::slice_stride(4 * p * (p - 1), block::team_threads(p));
 }
 
 // The dp4a product (every tap pair, whatever sm.dense_min).  The caller runs it with every thread of the crew, between
 // two barriers of the crew, after setup_quartic; consecutive products have degrees four apart or start again at degree 4 (their
-// unit counters alternate); ring: block_ring_words words, 16-byte aligned.
-template <int P, bool LAST, bool DEBUG>
+// unit counters alternate); ring: block_ring_words words, 16-byte aligned.  SMALL: the product's degree is 4P at most.
+template <int P, bool SMALL, bool LAST, bool DEBUG>
 __device__ __forceinline__ void block_chain_step(const uint32_t *__restrict__ in, uint32_t *__restrict__ out,
                                                  int m_in, Smem &sm, uint32_t *ring, const uint8_t *gs,
                                                  uint32_t *status, DebugPtrs dbg) {
-  block::run_strips<P, LAST, DEBUG>(in, out, m_in, sm, ring, gs, status, dbg);
+  constexpr bool kApart = SMALL && block::small_apart(P);
+  static_assert(kThreads / block::Ring<P, kApart>::team * block::Ring<P, kApart>::words <= block_ring_words(P),
+                "the small products' rings fit in the long ones'");
+  block::run_strips<P, kApart, LAST, DEBUG>(in, out, m_in, sm, ring, gs, status, dbg);
 }
 
 }  // namespace qfs

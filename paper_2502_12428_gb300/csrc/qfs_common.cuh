@@ -10,6 +10,7 @@ namespace qfs {
 constexpr int kThreads = 256;
 constexpr int kMaxUparDecl = 8;
 constexpr int kMaxStrips = 100;   // strips of a block product (qfs_block.cuh)
+constexpr int kMaxSmallStrips = 6;   // strips of one up to f~^p
 
 // Workspace buffers.  Every buffer a chain product reads from is preceded by kGuardWords zero words (the swept
 // product reads columns that do not exist from there).  A launch's workspace holds, per CTA, two buffers of
@@ -86,6 +87,7 @@ struct Smem {
     uint16_t chunk_tab[32 * 40];      // slice ring: flat chunk index -> (column - s0) << 8 | chunk
     struct {                          // block products
       uint32_t strip_tab[kMaxStrips]; // first item of every strip (block::build_strip_tab)
+      uint32_t small_tab[kMaxSmallStrips];   // the same of the products up to f~^p, where they have strips of their own
       int unit_next[2];               // next unit of a product's queue, by the product's parity
       int unit_slot[4][2];            // a team's next unit
     };

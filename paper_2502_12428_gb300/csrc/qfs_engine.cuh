@@ -465,14 +465,15 @@ __device__ __forceinline__ void ring_chain_step(const uint32_t *__restrict__ in,
 
 // One product of the chain: over the shared-memory slice ring above (int8 tensor form), by strips and blocks of slices
 // (qfs_block.cuh; dp4a form), or lane by lane over the input slices in global memory (qfs_sweep.cuh; int32 form).
-template <int P, int FORM, bool LAST, bool DEBUG>
+// SMALL: the product's degree is 4P at most.
+template <int P, int FORM, bool SMALL, bool LAST, bool DEBUG>
 __device__ __forceinline__ void chain_step(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, int m_in,
                                            Smem &sm, uint32_t *ring, const uint8_t *gs, uint32_t *status,
                                            DebugPtrs dbg) {
   if constexpr (uses_ring_chain(FORM, P))
     ring_chain_step<P, FORM, LAST, DEBUG>(in, out, m_in, sm, ring, gs, status, dbg);
   else if constexpr (FORM == 1)
-    block_chain_step<P, LAST, DEBUG>(in, out, m_in, sm, ring, gs, status, dbg);
+    block_chain_step<P, SMALL, LAST, DEBUG>(in, out, m_in, sm, ring, gs, status, dbg);
   else
     sweep_chain_step<P, LAST, DEBUG>(in, out, m_in, sm, gs, status, dbg);
 }
@@ -1145,7 +1146,7 @@ __device__ __noinline__ bool theta_poly(const uint32_t *__restrict__ dc, const u
 template <int P, int FORM, bool DEBUG>
 __device__ __noinline__ void chain_step_call(const uint32_t *in, uint32_t *out, int m_in, Smem &sm, uint32_t *ring,
                                              const uint8_t *gs, uint32_t *status, DebugPtrs dbg) {
-  chain_step<P, FORM, false, DEBUG>(in, out, m_in, sm, ring, gs, status, dbg);
+  chain_step<P, FORM, true, false, DEBUG>(in, out, m_in, sm, ring, gs, status, dbg);
 }
 
 // Tap words and the mask of nonzero pairs from sm.taps, by the first warp; the caller synchronises before and after.
@@ -1163,7 +1164,7 @@ __device__ __forceinline__ void build_tap_words(Smem &sm) {
 }
 
 // A1: read the 35 coefficients into the tap tables; returns false (after a barrier) if one is >= p.
-template <int P>
+template <int P, int FORM>
 __device__ __forceinline__ bool setup_quartic(const uint8_t *__restrict__ f35, Smem &sm) {
   using Pr = Prime<P>;
   const int tid = threadIdx.x;
@@ -1173,8 +1174,10 @@ __device__ __forceinline__ bool setup_quartic(const uint8_t *__restrict__ f35, S
     bad = a >= P;
     sm.taps[tid] = a;
   }
-  block::build_strip_tab(P, sm);
-  if (tid < 2) sm.unit_next[tid] = 0;
+  if constexpr (uses_blocks(FORM)) {
+    block::build_strip_tab(P, sm);
+    if (tid < 2) sm.unit_next[tid] = 0;
+  }
   if (__syncthreads_or(bad)) return false;
   build_tap_words(sm);
   if (tid >= 32 && tid < 32 + P) {
@@ -1232,12 +1235,12 @@ __device__ __forceinline__ void power_to_G(Smem &sm, const uint8_t *gs, uint32_t
   uint32_t *nxt = other;
   int m = Pr::d;
   for (int k = P - 1; k <= P * (P - 1) - 2; ++k) {
-    chain_step<P, FORM, false, DEBUG>(cur, nxt, m, sm, ring, gs, status, dbg);
+    chain_step<P, FORM, false, false, DEBUG>(cur, nxt, m, sm, ring, gs, status, dbg);
     crew_sync(sm.crew);
     uint32_t *t = cur; cur = nxt; nxt = t;
     m += 4;
   }
-  chain_step<P, FORM, LAST_DELTA, DEBUG>(cur, last_out ? last_out : nxt, m, sm, ring, gs, status, dbg);
+  chain_step<P, FORM, false, LAST_DELTA, DEBUG>(cur, last_out ? last_out : nxt, m, sm, ring, gs, status, dbg);
   crew_sync(sm.crew);
 }
 
@@ -1600,7 +1603,7 @@ __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem 
   using Pr = Prime<P>;
   const int tid = threadIdx.x;
   theta_steps = 0;
-  if (!setup_quartic<P>(f35, sm)) return -1;
+  if (!setup_quartic<P, FORM>(f35, sm)) return -1;
   uint32_t *cur = power_to_g<P, FORM, DEBUG>(sm, gs, ring, bufA, bufB, status, dbg);
   uint32_t *other = cur == bufA ? bufB : bufA;
   if (DEBUG)

@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kThreads, 2) stage_fedder(StagedChunk c) {
     __syncthreads();
     const int row = (int)sm->item;
     if (row >= c.n) break;
-    if (!setup_quartic<P>(c.coeffs + 35 * (size_t)row, *sm)) {
+    if (!setup_quartic<P, kForm>(c.coeffs + 35 * (size_t)row, *sm)) {
       if (threadIdx.x == 0) c.heights[row] = -1;
       continue;
     }
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kThreads, 2) stage_power(StagedChunk c) {
     __syncthreads();
     const unsigned slot = (unsigned)sm->item;
     if (slot >= total) break;
-    setup_quartic<P>(c.coeffs + 35 * (size_t)c.rows[slot], *sm);
+    setup_quartic<P, kForm>(c.coeffs + 35 * (size_t)c.rows[slot], *sm);
     uint32_t *cur = power_to_g<P, kForm, false>(*sm, gs, ring, bufA, bufB, c.status, dbg);
     for (int i = threadIdx.x; i < Pr::ld; i += blockDim.x) c.gA[(size_t)slot * Pr::ld + i] = gs[i];
     power_to_G<P, kForm, false, false>(*sm, gs, ring, cur, cur == bufA ? bufB : bufA, c.G + slot * gwords,

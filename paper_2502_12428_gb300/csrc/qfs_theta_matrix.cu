@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(kThreads, 2) theta_delta_kernel(const uint8_t 
   __syncthreads();
   DebugPtrs dbg{nullptr, nullptr, nullptr, nullptr};
   const int crew = crew_size(), rank = crew_rank(), q = (int)blockIdx.x / crew;
-  if (!setup_quartic<P>(coeffs + 35 * (size_t)q, sm)) {   // the same for the whole crew
+  if (!setup_quartic<P, QFS_FORM_DP4A>(coeffs + 35 * (size_t)q, sm)) {   // the same for the whole crew
     if (threadIdx.x == 0 && rank == 0) which[q] = -1;   // a coefficient >= p: M is left zero
     return;
   }

@@ -147,6 +147,34 @@ def test_dp4a_product_tap_positions(qfs, p, step):
     assert qfs.read_status() == 0
 
 
+@pytest.mark.parametrize("p", [3, 5, 7, 11, 13])
+def test_dp4a_small_products(qfs, p):
+    # f^(p-1) mod p by the products up to degree 4(p - 1), element by element, on quartics whose taps sit alone in the dp4a
+    # windows and on random ones; and f~^p mod p^2 by the identity and reduced modes' heights
+    def power(f, n):
+        form = {m: int(c) for m, c in zip(oracle.form_monomials(4), f) if c}
+        side = 4 * n + 1
+        out = np.zeros((side,) * 3, np.int64)
+        out[0, 0, 0] = 1
+        for _ in range(n):
+            prev, out = out, np.zeros_like(out)
+            for (_, a, b, c), v in form.items():
+                out[a:, b:, c:] += v * prev[:side - a, :side - b, :side - c]
+            out %= p
+        return np.array([out[e[1:]] for e in oracle.form_monomials(4 * n)])
+    rows = _edge_quartics(p)[::3] + list(inputs.dense(p, 4, 9300 + p))
+    for f in rows:
+        got = qfs.debug_stages(p, dev_tensor(f), max_h=2, power="reduced")
+        assert np.array_equal(got["g"].cpu().numpy(), power(f, p - 1))
+    assert np.array_equal(gpu_heights(qfs, p, np.stack(rows), power="reduced"), oracle.heights(p, np.stack(rows)))
+    if p >= 11:   # a light prime in the same launch: its own strips, and the first prime's again
+        other = inputs.sparse(5, 50, 9310)
+        outs = qfs.heights_multi([(5, dev_tensor(other), None), (p, dev_tensor(np.stack(rows)), None)], power="reduced")
+        assert np.array_equal(outs[0].cpu().numpy(), oracle.heights(5, other))
+        assert np.array_equal(outs[1].cpu().numpy(), oracle.heights(p, np.stack(rows)))
+    assert qfs.read_status() == 0
+
+
 # ------------------------------------------------------------------------------------- heights, small sets
 @pytest.mark.parametrize("form", CORE_FORMS)
 def test_heights_p3_64_plus_fermat(qfs, form):
