@@ -22,7 +22,7 @@ namespace {
 // Fixed scratch per device: 64 MiB.  Bytes [0, 256) are the control block: the work-queue counter at 0 (cleared
 // by every call), the device check word at 8 and the two work counters at 16 (both accumulate across calls until
 // qfs_read_status / qfs_read_stats take and clear them); the rest holds the two ping-pong buffers of every
-// persistent CTA.
+// persistent CTA and, where they all fit, its residue classes of theta.
 constexpr size_t kScratchBytes = size_t(64) << 20;
 constexpr size_t kControlBytes = 256;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -147,6 +147,13 @@ extern "C" int qfs_heights_noalloc(int p, int64_t n, const uint8_t *coeffs, int 
   prm.stats = reinterpret_cast<unsigned long long *>(base + 16);
   prm.ws = reinterpret_cast<uint32_t *>(base + kControlBytes);
   prm.ws_words = ws_words;
+  // theta by rows where every CTA's classes fit beside its buffers (p = 3; 2,000 quartics take 284 us by cubes, 216 us so)
+  const size_t ws_end = (kControlBytes + workspace_words(grid, ws_words) * sizeof(uint32_t) + 15) & ~size_t(15);
+  const size_t class_words = theta_by_rows(p, QFS_POWER_CHAIN) ? row_class_words(p) : 0;
+  if (class_words && ws_end + (size_t)grid * class_words * sizeof(uint32_t) <= kScratchBytes) {
+    prm.classes = reinterpret_cast<uint32_t *>(base + ws_end);
+    prm.class_words = class_words;
+  }
   prm.crew = 1;
   prm.crews[0] = 1;
   prm.power_mode = QFS_POWER_CHAIN;

@@ -357,6 +357,17 @@ def test_theta_by_rows_many_steps(qfs, p, n, form):
     assert qfs.read_status() == 0
 
 
+@pytest.mark.parametrize("p,n", [(3, 1), (3, 5000), (5, 1), (5, 130), (5, 140), (5, 3000)])
+def test_noalloc_theta_by_rows_and_by_cubes(qfs, p, n):
+    # in the fixed 64 MiB: classes by rows where every CTA's fit (p = 3; p = 5 up to about 136 quartics), cubes otherwise
+    f = inputs.sparse(p, n, 9950 + p)
+    want = oracle.heights(p, f)
+    t = dev_tensor(f)
+    for _ in range(2):
+        assert np.array_equal(qfs.heights_noalloc(p, t).cpu().numpy(), want)
+    assert qfs.read_status() == 0
+
+
 @pytest.mark.parametrize("p,n", [(3, 3000), (5, 4000), (7, 600)])
 @pytest.mark.parametrize("form", CORE_FORMS)
 def test_identity_theta_by_rows(qfs, p, n, form):
