@@ -1236,12 +1236,12 @@ __device__ __forceinline__ void power_to_G(Smem &sm, const uint8_t *gs, uint32_t
   int m = Pr::d;
   for (int k = P - 1; k <= P * (P - 1) - 2; ++k) {
     chain_step<P, FORM, false, false, DEBUG>(cur, nxt, m, sm, ring, gs, status, dbg);
-    crew_sync(sm.crew);
+    crew_sync(FORM == 1 ? sm.crew : 1);
     uint32_t *t = cur; cur = nxt; nxt = t;
     m += 4;
   }
   chain_step<P, FORM, false, LAST_DELTA, DEBUG>(cur, last_out ? last_out : nxt, m, sm, ring, gs, status, dbg);
-  crew_sync(sm.crew);
+  crew_sync(FORM == 1 ? sm.crew : 1);
 }
 
 // The identity power mode at p <= 7, by residue classes: Delta_1(f^(p-1)) = E(x^p) - f^(p-2)(x^p) Delta_1(f) (mod p)
@@ -1661,7 +1661,7 @@ __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem 
   } else {
     delta_to_guarded<P>(delta, dg, sm);
   }
-  crew_sync(sm.crew);
+  crew_sync(FORM == 1 ? sm.crew : 1);
   uint8_t *g = gs, *g2 = gn;
   for (int h = 2; h <= max_h; ++h) {
     bool nonzero;
@@ -1681,6 +1681,32 @@ __device__ int process_quartic(const uint8_t *__restrict__ f35, int max_h, Smem 
     __syncthreads();
   }
   return 0;
+}
+
+// process_quartic in a fused launch.  In the forms whose products are part of it (int8 tensor) or call it often with many
+// registers (int32) it is a function of its own, so that the queue around it takes none of its registers: 8,192 quartics
+// at p = 7 in the int8 tensor form take 87.7 ms, inlined 90.4.  The dp4a form is faster inlined (sparse p = 5: 15.6 and 15.8).
+template <int P, int FORM>
+__device__ __noinline__ int process_quartic_apart(const uint8_t *__restrict__ f35, int max_h, Smem &sm, uint8_t *gs,
+                                                  uint8_t *gn, uint32_t *ring, uint32_t *bufA, uint32_t *bufB,
+                                                  uint32_t *status, int &theta_steps, int power_mode,
+                                                  uint32_t *classes) {
+  return process_quartic<P, FORM, false>(f35, max_h, sm, gs, gn, ring, bufA, bufB, status,
+                                         DebugPtrs{nullptr, nullptr, nullptr, nullptr}, theta_steps, power_mode, nullptr,
+                                         classes);
+}
+template <int P, int FORM>
+__device__ __forceinline__ int fused_quartic(const uint8_t *__restrict__ f35, int max_h, Smem &sm, uint8_t *gs,
+                                             uint8_t *gn, uint32_t *ring, uint32_t *bufA, uint32_t *bufB,
+                                             uint32_t *status, int &theta_steps, int power_mode, uint32_t *crewA,
+                                             uint32_t *classes) {
+  if constexpr (FORM == 1)
+    return process_quartic<P, FORM, false>(f35, max_h, sm, gs, gn, ring, bufA, bufB, status,
+                                           DebugPtrs{nullptr, nullptr, nullptr, nullptr}, theta_steps, power_mode, crewA,
+                                           classes);
+  else
+    return process_quartic_apart<P, FORM>(f35, max_h, sm, gs, gn, ring, bufA, bufB, status, theta_steps, power_mode,
+                                          classes);
 }
 
 // ------------------------------------------------------------------------------------------------ fused launch
@@ -1794,7 +1820,6 @@ __device__ __forceinline__ void fused_body(const FusedParams &prm) {
   init_task_queue(sm);
   uint32_t *bufA, *bufB;
   cta_buffers(prm.ws, prm.ws_words, bufA, bufB);
-  DebugPtrs dbg{nullptr, nullptr, nullptr, nullptr};
   const int crew = FORM == 1 ? prm.crew : 1, rank = crew > 1 ? crew_rank() : 0;
   uint32_t *classes = prm.classes ? prm.classes + (size_t)blockIdx.x * prm.class_words : nullptr;
   uint32_t *first = bufA - (size_t)rank * 2 * prm.ws_words;   // the crew's first buffer
@@ -1841,16 +1866,16 @@ __device__ __forceinline__ void fused_body(const FusedParams &prm) {
     const uint8_t *f = G.coeffs + 35 * row;
     int h, steps;
     switch (G.p) {
-      case 3: h = process_quartic<3, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA, classes); break;
-      case 5: h = process_quartic<5, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA, classes); break;
+      case 3: h = fused_quartic<3, FORM>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, steps, prm.power_mode, crewA, classes); break;
+      case 5: h = fused_quartic<5, FORM>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, steps, prm.power_mode, crewA, classes); break;
       default:
         if constexpr (SMALL) {
           h = -1;   // not reached: the host launches the small-prime kernel only when every group has p <= 5
         } else {
           switch (G.p) {
-            case 7: h = process_quartic<7, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA, classes); break;
-            case 11: h = process_quartic<11, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA, classes); break;
-            default: h = process_quartic<13, FORM, false>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, dbg, steps, prm.power_mode, crewA, classes); break;
+            case 7: h = fused_quartic<7, FORM>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, steps, prm.power_mode, crewA, classes); break;
+            case 11: h = fused_quartic<11, FORM>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, steps, prm.power_mode, crewA, classes); break;
+            default: h = fused_quartic<13, FORM>(f, prm.max_h, sm, gs, gn, ring, bufA, bufB, prm.status, steps, prm.power_mode, crewA, classes); break;
           }
         }
         break;
