@@ -32,7 +32,8 @@ struct DeviceState {
   void *ws = nullptr;          // persistent-CTA workspaces
   size_t ws_bytes = 0;
   void *ctrl = nullptr;        // [8]: status (u32), [16]: stats (2 x u64); cleared by every fused launch: [32]: work counters
-                               // (2 x u64), [48]: survivors of every group (QFS_MAX_GROUPS x u64)
+                               // (2 x u64), [48]: survivors of every group and its
+                               // first item (2 x QFS_MAX_GROUPS x u64)
   void *staged = nullptr;      // staged-engine survivor buffers
   size_t staged_bytes = 0;
   int *which = nullptr;        // theta-matrix export: which workspace buffer holds each quartic's Delta
@@ -46,7 +47,7 @@ struct DeviceState {
   size_t list_bytes = 0;
 };
 
-constexpr size_t kControlBytes = 48 + 8 * QFS_MAX_GROUPS;
+constexpr size_t kControlBytes = 48 + 16 * QFS_MAX_GROUPS;
 constexpr int kMinRowBlock = 1024;   // rows of A that a mod-p product takes at least at once, whatever the memory
 constexpr int kMaxDevices = 64;
 DeviceState g_dev[kMaxDevices];
@@ -442,6 +443,7 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
   prm.status = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(S->ctrl) + 8);
   prm.stats = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(S->ctrl) + 16);
   const bool one_prime = same_prime(prm);
+  prm.grouped = !one_prime;
   // the reduced mode of one small prime (dp4a form) has a kernel of its own, which needs no workspace (so no budget is
   // too small for it); a call that caps the CTAs or mixes primes takes the fused kernel
   const bool reduced = power == QFS_POWER_REDUCED && form == QFS_FORM_DP4A && max_p <= kReducedMaxP && one_prime &&
@@ -474,7 +476,7 @@ int qfs_heights_multi_ex(int n_groups, const qfs_group_t *groups, int max_h, con
   // height-1 screen first: the persistent launch then runs only the quartics that pass it
   rc = ensure_list(*S, (size_t)n_items * sizeof(int64_t));
   if (rc) return rc;
-  cudaError_t e = cudaMemsetAsync(prm.counter, 0, (2 + QFS_MAX_GROUPS) * sizeof(unsigned long long), stream);
+  cudaError_t e = cudaMemsetAsync(prm.counter, 0, (2 + 2 * QFS_MAX_GROUPS) * sizeof(unsigned long long), stream);
   if (e != cudaSuccess) return cuda_fail(e);
   const int64_t screen_ctas = std::min<int64_t>((n_items + 7) / 8, (int64_t)S->sms * 8);
   e = screen_launch(prm, max_p, static_cast<int64_t *>(S->list), n_list, (int)screen_ctas, stream);

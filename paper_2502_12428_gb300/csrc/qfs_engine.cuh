@@ -1740,23 +1740,29 @@ struct FusedParams {
                                       // launch over several primes with crews is the only one: crews[0] is 0
   int crew_rounds;                    // quartics of one prime that a crew of 2 or more may take one after another
   int power_mode;                     // 0: chain (Algorithm 1 literally), 1: identity shortcut, 2: reduced theta
-  const int64_t *list;                // if set: the items to run (the survivors of the height-1 screen), every group's
-                                      // from its item_begin on ...
-  const unsigned long long *n_list;   // ... and their count for each group; if null, every item 0 .. n_items-1 runs
+  const int64_t *list;                // if set: the items to run, the survivors of the height-1 screen ...
+  const unsigned long long *n_list;   // ... and their count; if null, every item 0 .. n_items-1 runs
+  int grouped;                        // the survivors are listed group by group: those of group g from list[begin] on,
+                                      // n_list[g] of them, with begin = n_list[kMaxGroups + g]
 };
 
-// Item k of those to run, group after group (the largest prime first).
-__device__ __forceinline__ int64_t listed_item(const FusedParams &prm, int64_t k) {
-  if (!prm.list) return k;
-  int g = 0;
-  for (; g + 1 < prm.n_groups && k >= (int64_t)prm.n_list[g]; ++g) k -= (int64_t)prm.n_list[g];
-  return prm.list[prm.g[g].item_begin + k];
-}
+// Items to run.
 __device__ __forceinline__ int64_t listed_items(const FusedParams &prm) {
   if (!prm.list) return prm.n_items;
-  int64_t n = 0;
-  for (int g = 0; g < prm.n_groups; ++g) n += (int64_t)prm.n_list[g];
+  int64_t n = (int64_t)prm.n_list[0];
+  if (prm.grouped)
+    for (int g = 1; g < prm.n_groups; ++g) n += (int64_t)prm.n_list[g];
   return n;
+}
+// Item k of those to run; with groups, group after group (the largest prime first).
+inline __device__ __noinline__ int64_t grouped_item(const int64_t *list, const unsigned long long *n_list, int64_t k) {
+  int g = 0;
+  for (; g + 1 < kMaxGroups && k >= (int64_t)n_list[g]; ++g) k -= (int64_t)n_list[g];
+  return list[(int64_t)n_list[kMaxGroups + g] + k];
+}
+__device__ __forceinline__ int64_t listed_item(const FusedParams &prm, int64_t k) {
+  if (!prm.list) return k;
+  return prm.grouped ? grouped_item(prm.list, prm.n_list, k) : prm.list[k];
 }
 
 // The crew size for n_run quartics of one prime, among those that launches are made for.  Crews of 8 while each quartic

@@ -215,12 +215,12 @@ __global__ void __launch_bounds__(kRThreads) reduced_kernel(const __grid_constan
       S.powp[threadIdx.x] = v;
     }
   }
-  const int64_t n_run = listed_items(prm);
+  const int64_t n_run = (int64_t)*prm.n_list;
   for (;;) {
     __syncthreads();
     if (threadIdx.x == 0) {
       const int64_t k = (int64_t)atomicAdd(prm.counter, 1ull);
-      S.item = k < n_run ? listed_item(prm, k) : -1;
+      S.item = k < n_run ? prm.list[k] : -1;
     }
     __syncthreads();
     const int64_t item = S.item;

@@ -96,6 +96,8 @@ __global__ void __launch_bounds__(kScreenThreads) screen_kernel(const __grid_con
   uint16_t *items = reinterpret_cast<uint16_t *>(smem);
   uint32_t *wsm = smem + screen_item_words(max_p) + (size_t)warp * screen_warp_words(max_p);
   rows::build_items(items, 2 * (max_p - 1));
+  if (blockIdx.x == 0 && (int)threadIdx.x < prm.n_groups)
+    n_list[kMaxGroups + threadIdx.x] = (unsigned long long)prm.g[threadIdx.x].item_begin;
   __syncthreads();
   const int64_t stride = (int64_t)gridDim.x * kScreenWarps;
   int last_p = 0;   // prime of the forms in the warp's region
@@ -117,7 +119,8 @@ __global__ void __launch_bounds__(kScreenThreads) screen_kernel(const __grid_con
     }
     if (lane == 0) {
       if (r != 0) G.heights[row] = (int8_t)r;
-      else list[G.item_begin + (int64_t)atomicAdd(n_list + gi, 1ull)] = item;
+      else if (prm.grouped) list[G.item_begin + (int64_t)atomicAdd(n_list + gi, 1ull)] = item;
+      else list[atomicAdd(n_list, 1ull)] = item;
     }
     __syncwarp();
   }
