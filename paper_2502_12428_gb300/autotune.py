@@ -3,9 +3,9 @@
 Per prime it times the fused engine on seeded random quartics and keeps the fastest candidate of two shapes:
 - ring: the tile of the shared-memory slice ring that the int8 tensor form's chain runs over (work items per
   round x shared-memory ring size);
-- sweep: the launch shape of the swept chain of the dp4a and int32 forms (the nonzero tap pairs from which a
-  quartic runs every pair in the two-slice loop, and the CTAs per SM).  Its sample is half dense and half sparse
-  quartics, since the threshold decides between the two paths only for quartics with zero coefficients.
+- sweep: the launch shape of the dp4a and int32 forms: the CTAs per SM and, for the int32 form, the nonzero tap pairs
+  from which a quartic's products run every pair.  Its sample is half dense and half sparse quartics, since the
+  threshold matters only for quartics with zero coefficients.
 It writes paper_2502_12428_gb300/tile_table.json, which the Python binding applies when it loads the library.
 Heights do not depend on any of these shapes.
 """

@@ -672,6 +672,7 @@ int qfs_sweep_autotune(int form, int p, int64_t n, const uint8_t *coeffs, int *b
   cudaEventCreate(&a);
   cudaEventCreate(&b);
   const int dense[] = {0, 6, 8, 10, 12, 14, 16};
+  const int n_dense = form == QFS_FORM_INT32 ? 7 : 1;   // the dp4a product has no threshold: its default stays
   SweepConfig &slot = g_sweep[form == QFS_FORM_DP4A][p];
   const SweepConfig saved = slot;
   // the CTAs per SM that fit: the occupancy of the launch a default shape would make
@@ -691,9 +692,9 @@ int qfs_sweep_autotune(int form, int p, int64_t n, const uint8_t *coeffs, int *b
   opt.engine = QFS_ENGINE_FUSED;
   opt.power = QFS_POWER_CHAIN;
   qfs_group_t g{p, n, coeffs, out};
-  for (int dm : dense)
+  for (int di = 0; di < n_dense; ++di)
     for (int c = 1; c <= max_ctas && rc == QFS_OK; ++c) {
-      slot = SweepConfig{dm, c};
+      slot = SweepConfig{dense[di], c};
       rc = qfs_heights_multi_ex(1, &g, 10, &opt, 0);  // warm-up
       if (rc) break;
       float ms = 1e30f;

@@ -80,7 +80,7 @@ struct Smem {
   int taps[35];           // coefficients of f, packed order (index tet(uI) + tri(sI) + tI)
   uint32_t tapword[15];   // tap words per (uI, sI) pair: byte k = a(uI, sI, 3-k)
   uint32_t pair_mask;     // bit tri(uI)+sI set iff that pair has a nonzero tap
-  int dense_min;          // nonzero tap pairs from which the swept chain runs every pair (the two-slice loop)
+  int dense_min;          // nonzero tap pairs from which the swept chain (int32 form) runs every pair
   int powp[kMaxP];        // c^p mod p^2
   int slot_tab[2][kMaxUparDecl + 4];  // ring word offsets of the slices a chain round reads (double buffered)
   union {                             // one product form per launch

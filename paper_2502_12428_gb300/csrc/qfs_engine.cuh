@@ -52,7 +52,7 @@ struct TileConfig {
   int ring_words;
 };
 
-// Swept-chain launch shape of one prime and form (dp4a, int32): dense_min = nonzero tap pairs (of 15) from which
+// Launch shape of one prime and form (dp4a, int32): dense_min (int32 only) = nonzero tap pairs (of 15) from which
 // a quartic takes the every-pair path (16: never), ctas_per_sm = CTAs per SM of the fused launch (0: as many as
 // fit).  Results never depend on either.
 constexpr int kDefaultDenseMin = 12;

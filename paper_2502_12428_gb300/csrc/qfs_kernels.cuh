@@ -6,8 +6,8 @@
 
 namespace qfs {
 
-// Resident CTAs per SM the register allocation is bounded for: the swept chain (dp4a and int32 forms) keeps five
-// accumulator sets per lane and gets 128 registers (2 CTAs of 256 threads); the int8 tensor form gets 85 (3 CTAs).
+// Resident CTAs per SM the register allocation is bounded for: the products of the dp4a and int32 forms keep four or five
+// accumulator sets per lane and get 128 registers (2 CTAs of 256 threads); the int8 tensor form gets 85 (3 CTAs).
 template <int FORM>
 constexpr int min_ctas_per_sm() { return FORM == 2 ? 3 : 2; }
 // Persistent launch: every CTA pulls quartics from a global atomic queue until the queue is empty.

@@ -294,7 +294,7 @@ def _form_id(form):
 
 
 def sweep_tune_set(form, p, dense_min, ctas_per_sm):
-    """qfs_sweep_tune_set: swept-chain shape of (form, p); (0, 0) restores the defaults."""
+    """qfs_sweep_tune_set: launch shape of (form, p); (0, 0) restores the defaults."""
     _check(_lib().qfs_sweep_tune_set(_form_id(form), int(p), int(dense_min), int(ctas_per_sm)), "qfs_sweep_tune_set")
 
 
@@ -305,7 +305,7 @@ def sweep_tune_get(form, p):
 
 
 def sweep_autotune(p, sample, form="dp4a"):
-    """Times every candidate swept-chain shape (dense threshold x CTAs per SM) on `sample` (CUDA uint8 n x 35) and
+    """Times every candidate launch shape (CTAs per SM; int32 form: times the threshold) on `sample` (CUDA uint8 n x 35) and
     keeps the fastest for (form, p)."""
     _need_cuda(sample, torch.uint8, "sample")
     dm, c, ms = ctypes.c_int(0), ctypes.c_int(0), ctypes.c_float(0)
@@ -316,7 +316,7 @@ def sweep_autotune(p, sample, form="dp4a"):
 
 def load_tile_table(path=TILE_TABLE):
     """Applies a persisted tile table (missing file: nothing to do): per prime the ring tile of the int8 tensor
-    form, and under "sweep" the swept-chain shape of each of the dp4a and int32 forms.  Returns the entries."""
+    form, and under "sweep" the launch shape of the dp4a and int32 forms.  Returns the entries."""
     import json
     if not os.path.exists(path):
         return {}

@@ -145,6 +145,11 @@ int noalloc_take_counters(uint32_t *, unsigned long long *) { return 0; }
 #define cudaFree(p) fake::release(p)
 #define cudaMemset(p, v, n) ((void)(p), cudaSuccess)
 #define cudaMemsetAsync(p, v, n, s) ((void)(p), cudaSuccess)
+#define cudaEventCreate(e) ((void)(e), cudaSuccess)
+#define cudaEventDestroy(e) ((void)(e), cudaSuccess)
+#define cudaEventRecord(e, s) ((void)(e), cudaSuccess)
+#define cudaEventSynchronize(e) ((void)(e), cudaSuccess)
+#define cudaEventElapsedTime(ms, a, b) (*(ms) = 1.f, cudaSuccess)
 #include "qfs_api.cu"
 
 namespace {
@@ -199,6 +204,12 @@ int main(int argc, char **argv) {
         n_list[n] = (unsigned long long)num(("n" + std::to_string(n + 1)).c_str(), 0);
       }
       rc = (int)joint_items(n, g, n_list, (int)num("crew", 8), num("ctas", 304), 3);
+    } else if (op == "sweep_autotune") {
+      int dense = -1, ctas = -1;
+      float ms = 0;
+      rc = qfs_sweep_autotune((int)num("form", QFS_FORM_DP4A), (int)num("p", 7), num("n", 1), rows, &dense, &ctas, &ms);
+      fake::record("best dense_min=%d ctas=%d", dense, ctas);
+      qfs_sweep_tune_set((int)num("form", QFS_FORM_DP4A), (int)num("p", 7), 0, 0);
     } else if (op == "prepare") {
       rc = qfs_plan_prepare((int)num("p", 7), num("n", 0));
     } else if (op == "theta_matrix") {

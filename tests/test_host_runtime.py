@@ -166,3 +166,12 @@ def test_two_ctas_per_sm_in_every_mode(runtime, p, power, form):
     if form == 0 and power == 2:   # nothing is staged: the iterates and the mode's byte arrays
         ld, fpm2, d1f = ((d + 1) * (d + 2) * (d + 3) // 6 for d in (4 * (p - 1), 4 * (p - 2), 4 * p))
         assert r["fused"][0]["smem"] <= 6000 + 2 * ld + fpm2 + d1f + 300
+
+
+@pytest.mark.parametrize("form,thresholds", [(0, 7), (1, 1)])
+def test_sweep_autotune_times_what_has_an_effect(runtime, form, thresholds):
+    # one warm-up and two timed launches for each shape; the dp4a product runs every tap pair whatever the threshold
+    r = runtime(op="sweep_autotune", form=form, p=5, n=20000)
+    assert r["rc"] == 0
+    assert r["launches"].count("screen") == 3 * thresholds * 2 and len(r["fused"]) == 3 * thresholds * 2
+    assert r["launches"][-1].startswith("best dense_min=0 ")
