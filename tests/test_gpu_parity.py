@@ -758,6 +758,46 @@ def test_matmul_mod_unaligned_views(qfs):
         assert not bufs[2][:off].any() and not bufs[2][off + n * m:].any()
 
 
+@pytest.mark.parametrize("p,top", [(33, 16), (31, 15), (29, 14), (34, 17), (101, 50), (129, 64), (251, 125), (255, 127),
+                                   (256, 128)])
+@pytest.mark.parametrize("steps_past", [0, 1])
+@pytest.mark.parametrize("constant", [False, True])
+def test_matmul_mod_at_the_float32_bound(qfs, p, top, steps_past, constant):
+    # Residues are taken in the symmetric range, so operands of one sign next to p / 2 make the largest sums, up to 2^24 at
+    # p = 33, and odd values next to them the ones whose last bit counts.  A drain comes after `steps` K steps of 128;
+    # K is one drain, and one drain and a step.
+    mag = p // 2 if p <= 33 else p // 2 + 16
+    steps = 2 ** 24 // (mag * mag * 128)
+    k = 128 * (steps + steps_past)
+    n, m = (130, 260) if k <= 20000 else (37, 41)
+    rng = np.random.default_rng(1000 * p + k)
+    A, B = (np.full(s, top, np.uint8) if constant else rng.integers(top - 1, top + 1, s, dtype=np.uint8)
+            for s in ((n, k), (k, m)))
+    A[0, ::7] = top - 1
+    drained = A[:, :128 * steps].astype(np.float64) @ B[:128 * steps].astype(np.float64)
+    limit = top * top * 128 * steps
+    assert limit == 2 ** 24 or p != 33
+    assert drained.max() > 0.9 * limit and drained.max() <= 2 ** 24
+    got = qfs.matmul_mod(p, dev_tensor(A), dev_tensor(B)).cpu().numpy()
+    want = A.astype(np.float64) @ B.astype(np.float64) % p   # sums below 2^53
+    assert np.array_equal(got, want.astype(np.uint8))
+    assert qfs.read_status() == 0
+
+
+@pytest.mark.parametrize("p,top", [(251, 125), (33, 16), (11, 5)])
+def test_matmul_mod_sums_past_float32(qfs, p, top):
+    # a long K whose undrained sum leaves the integers that float32 holds: 2^29 at p = 251, 2^26 at p = 33
+    k = {251: 40000, 33: 300000, 11: 3000000}[p]
+    rng = np.random.default_rng(p)
+    A = rng.integers(max(top - 19, top // 2), top + 1, (16, k), dtype=np.uint8)
+    B = rng.integers(max(top - 19, top // 2), top + 1, (k, 24), dtype=np.uint8)
+    want = A.astype(np.float64) @ B.astype(np.float64)
+    assert want.max() > 1.5 * 2 ** 24
+    got = qfs.matmul_mod(p, dev_tensor(A), dev_tensor(B)).cpu().numpy()
+    assert np.array_equal(got, (want % p).astype(np.uint8))
+    assert qfs.read_status() == 0
+
+
 @pytest.mark.parametrize("p", [11, 251])
 @pytest.mark.parametrize("n,m", [(1, 1), (31, 3), (33, 255), (127, 257), (129, 258), (161, 511), (200, 515)])
 def test_matmul_mod_rows_at_odd_addresses(qfs, p, n, m):
