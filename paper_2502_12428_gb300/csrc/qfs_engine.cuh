@@ -1770,6 +1770,9 @@ __device__ __forceinline__ int64_t listed_item(const FusedParams &prm, int64_t k
 // call by crews of 1, 2, 4 and 8; 304, 152, 76 and 38 run at once):
 //     36: 3.7, 2.1, 1.2, 1.0     100: 3.7, 2.8, 2.4, 2.7     160: 5.1, 4.1, 3.6, 4.1     250: 5.3, 5.2, 4.9, 6.0
 //     310: 7.0, 6.3, 6.1, 7.3    400: 8.0, 7.6, 7.6, 9.4     600: 10.4, 10.6, 11.4, 13.8
+// and at p = 11, where the same counts serve:
+//     15: 129, 68, 37, 21        45: 134, 70, 48, 44         110: 167, 106, 87, 89       230: 201, 186, 164, 171
+//     300: 214, 193, 213, 225    (p = 13: 16: 463, 242, 130, 80      70: 476, 246, 196, 206)
 // That is with two CTAs on every SM.  On a part of the device (a small workspace budget) a CTA has an SM to itself: one
 // quartic takes 2.8, 1.6, 1.0 and 0.6 ms, and crews are better only while each quartic gets one at once (`rounds` = 1; 3
 // quartics on 3 CTAs: 2.8 ms, by one crew of 2 4.7 ms).
