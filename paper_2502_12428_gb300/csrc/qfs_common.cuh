@@ -46,7 +46,8 @@ struct DebugPtrs {
 
 // Crews.  A launch over few quartics runs as thread-block clusters: the CTAs of a cluster (a crew, 1, 2, 4 or 8 of them)
 // work on one quartic together.  Each forms f^(p-1) for itself; the products of A4 and the theta steps are split, with
-// the forms in the first CTA's buffers.  Every CTA of a crew takes the same decisions from the same data.
+// the forms in the first CTA's buffers.  Every CTA of a crew takes the same decisions from the same data.  In a launch over
+// several primes the crews take the heavy quartics, then each CTA the rest for itself (joint_items in qfs_engine.cuh).
 #if defined(__CUDACC__)
 __device__ __forceinline__ int crew_rank() {
   unsigned r;

@@ -89,6 +89,9 @@ __device__ int screen_row(const uint8_t *__restrict__ f35, uint32_t *wsm, const 
   return (acc % P) != 0 ? 1 : 0;
 }
 
+// GROUPED: survivors are listed group by group (a kernel of its own: with both lists in one, a row at p = 11 takes 3 us
+// more).
+template <bool GROUPED>
 __global__ void __launch_bounds__(kScreenThreads) screen_kernel(const __grid_constant__ FusedParams prm, int max_p,
                                                                 int64_t *list, unsigned long long *n_list) {
   extern __shared__ __align__(16) uint32_t smem[];
@@ -96,7 +99,7 @@ __global__ void __launch_bounds__(kScreenThreads) screen_kernel(const __grid_con
   uint16_t *items = reinterpret_cast<uint16_t *>(smem);
   uint32_t *wsm = smem + screen_item_words(max_p) + (size_t)warp * screen_warp_words(max_p);
   rows::build_items(items, 2 * (max_p - 1));
-  if (blockIdx.x == 0 && (int)threadIdx.x < prm.n_groups)
+  if (GROUPED && blockIdx.x == 0 && (int)threadIdx.x < prm.n_groups)
     n_list[kMaxGroups + threadIdx.x] = (unsigned long long)prm.g[threadIdx.x].item_begin;
   __syncthreads();
   const int64_t stride = (int64_t)gridDim.x * kScreenWarps;
@@ -119,7 +122,7 @@ __global__ void __launch_bounds__(kScreenThreads) screen_kernel(const __grid_con
     }
     if (lane == 0) {
       if (r != 0) G.heights[row] = (int8_t)r;
-      else if (prm.grouped) list[G.item_begin + (int64_t)atomicAdd(n_list + gi, 1ull)] = item;
+      else if (GROUPED) list[G.item_begin + (int64_t)atomicAdd(n_list + gi, 1ull)] = item;
       else list[atomicAdd(n_list, 1ull)] = item;
     }
     __syncwarp();
@@ -135,9 +138,10 @@ size_t screen_smem_bytes(int max_p) {
 cudaError_t screen_launch(const FusedParams &prm, int max_p, int64_t *list, unsigned long long *n_list,
                           int grid_ctas, cudaStream_t st) {
   const size_t smem = screen_smem_bytes(max_p);
-  cudaError_t e = cudaFuncSetAttribute(screen_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const auto kernel = prm.grouped ? screen_kernel<true> : screen_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  screen_kernel<<<grid_ctas, kScreenThreads, smem, st>>>(prm, max_p, list, n_list);
+  kernel<<<grid_ctas, kScreenThreads, smem, st>>>(prm, max_p, list, n_list);
   return cudaGetLastError();
 }
 
