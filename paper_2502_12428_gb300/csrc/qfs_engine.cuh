@@ -1767,7 +1767,7 @@ __device__ __forceinline__ int64_t listed_item(const FusedParams &prm, int64_t k
 
 // The crew size for n_run quartics of one prime, among those that launches are made for.  Crews of 8 while each quartic
 // gets one at once, smaller ones for up to three rounds, as measured at p = 7 with random quartics of height >= 2 (ms per
-// call by crews of 1, 2, 4 and 8; 304, 152, 76 and 38 run at once):
+// call by crews of 1, 2, 4 and 8; 304, 152, 74 to 76 and 36 to 38 run at once, as the GPU's clusters of SMs allow):
 //     36: 3.7, 2.1, 1.2, 1.0     100: 3.7, 2.8, 2.4, 2.7     160: 5.1, 4.1, 3.6, 4.1     250: 5.3, 5.2, 4.9, 6.0
 //     310: 7.0, 6.3, 6.1, 7.3    400: 8.0, 7.6, 7.6, 9.4     600: 10.4, 10.6, 11.4, 13.8
 // and at p = 11, where the same counts serve:

@@ -12,7 +12,8 @@
 // kept reversed (byte j of row s: F[s - j]), so that a row's terms are a run of Delta_1(f) against a run of F; the rows
 // of Delta_1(f) have zero guards on both sides instead of bounds checks.
 //
-// Bound by the latency of its small stages (four CTAs of 56 KB per SM at p = 7).  262,144 dense quartics at p = 7, of
+// Bound by the latency of its small stages: four CTAs of 56 KB per SM at p = 7, so 16 warps, which issue in 61 % of the
+// cycles (per issue: fixed latency 2.2, branches 0.7, barrier 0.5); no DRAM traffic to speak of.  262,144 dense quartics at p = 7, of
 // which 37,224 reach it: 4.9 ms, against 13.8 ms in the fused kernel, where 256 threads with 128 registers and 92 KB run
 // the same stages through device memory.
 #include <cuda_runtime.h>
