@@ -9,7 +9,7 @@
 // of theta_poly takes a scatter of every class into the cube, a barrier per class and a byte load per MAC.)
 //
 // Bound by latency and barriers at 16 warps per SM: the fused launch over sparse quartics at p = 5, where theta and the
-// classes are half of it, issues in 54 % of the cycles (per issue: fixed latency 1.6, barrier 1.5, shared memory 0.8), the
+// classes are two fifths of it, issues in 54 % of the cycles (per issue: fixed latency 1.6, barrier 1.5, shared memory 0.8), the
 // identity mode's at p = 7 in 58 %; DRAM 3 and 15 %.  Whole calls, by cube and by rows: p = 5, 131,071 sparse quartics (4.4 steps each) 133.9 and
 // 102.4 ms; p = 5, 65,536 dense 25.1 and 21.6 ms; 65 quartics at p = 3, where up to ten steps follow each other, 93 and 66 us.
 // The identity mode at p = 7, 65,536 dense quartics (9,400 past height 1): 41.8 and 23.7 ms.
