@@ -238,7 +238,7 @@ int qfs_theta_matrix(int p, int64_t n, const uint8_t *coeffs, uint8_t *M_out, cu
    in [0, p), 2 <= p <= 256 (p need not be prime); all caller-owned.  Exact: the fp8 tensor cores multiply small
    integers that e4m3 holds exactly (two planes per matrix for p > 33), and float32 sums are reduced mod p before they
    could leave the integers float32 holds exactly.  Stream-ordered; may grow a library scratch buffer ((n + m) x k
-   bytes rounded up, twice that for p > 33) with cudaMalloc.  Returns QFS_OK or QFS_ERR_INVALID_P, QFS_ERR_INVALID_N, QFS_ERR_NULL,
+   bytes rounded up, twice that for p > 33) with cudaMalloc; where that does not fit, it takes A by blocks of rows.  Returns QFS_OK or QFS_ERR_INVALID_P, QFS_ERR_INVALID_N, QFS_ERR_NULL,
    QFS_ERR_NO_MEMORY, QFS_ERR_CUDA (nothing enqueued on error).  n = 0 or m = 0 is a no-op; k = 0 zeroes C. */
 int qfs_matmul_mod(int p, int n, int m, int k, const uint8_t *A, const uint8_t *B, uint8_t *C, cudaStream_t stream);
 
